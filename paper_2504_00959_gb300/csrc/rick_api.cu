@@ -196,6 +196,26 @@ bool use_split(const rick_params& p, int* n1, int* n2)
     return !(p.flags & RICK_FFT_2D) && p.n >= kSplitMinN;
 }
 
+// The two-pass transform of rick_strip.cu (row transforms of what is not empty,
+// then the whole column transform fused with the screen and the stack): n =
+// 1024, 2048, 4096 unless RICK_FFT_2D asks for cuFFT's 2D plan, and up to
+// kStripAmp.  Measured, with the split transform before it: 4096^2 x 32 planes
+// x 1e7 measurements 4.99 -> 3.52 ms per image, 8 channels of 2048^2 x 16
+// 5.70 -> 4.72 ms, 1024^2 x 16 x 1e6 0.358 -> 0.343 ms.  It needs a second buffer of a group's planes (strip order); where that does not fit,
+// the handle takes the split transform or the 2D plan instead.
+bool want_strip(const rick_params& p) { return strip_shape(p.n) && !(p.flags & RICK_FFT_2D); }
+
+// Grid correction multiplies the planes' rounding (~3e-7 of their RMS,
+// uncorrelated between pixels) by 1 / (c(x) c(y)), over the image by mean(1 /
+// c^2) in RMS: 167 for the Kaiser-Bessel kernel of support 7, 479 for support
+// 8, 800 for the Gaussian of support 6 and over 1e6 for wider Gaussians, whose
+// transform passes through zero inside the image.  Two transforms that round
+// differently then differ by that much: of the image, 7e-6 at 167 and 2e-5 at
+// 479 (6 planes of 4096^2, 3e4 measurements).  Up to kStripAmp the image is
+// well above its rounding whatever the transform; beyond, a handle keeps the
+// transform that it always had, so that its images stay the same.
+constexpr double kStripAmp = 300.0;
+
 rick_status get_plan(rick_handle h, int batch, cufftHandle* out, int kind = kPlan2D)
 {
     const int key = (kind << 24) | batch;
@@ -338,6 +358,115 @@ rick_status colfft_ready(rick_handle h)
     return RICK_OK;
 }
 
+// The tiles the strip transform reads and writes: those with entries in the
+// stored chunks (all of them when the chunks take more than one pass, which
+// accumulates onto every tile).
+bool skips_empty(rick_handle h) { return h->strip && h->chunks.size() <= (size_t)kMaxChunksPerPass; }
+
+ChunkList chunk_list(rick_handle h, size_t c0)
+{
+    ChunkList cl{};
+    for (size_t q = c0; q < h->chunks.size() && cl.count < kMaxChunksPerPass; ++q, ++cl.count) {
+        cl.off[cl.count] = h->chunks[q].off;
+        cl.ent[cl.count] = h->chunks[q].ent;
+    }
+    return cl;
+}
+
+// The w-screen constants of a single image's planes.
+StackArgs stack_args(rick_handle h)
+{
+    const rick_params& p = h->p;
+    const double dw = (p.nw > 1) ? (p.w_max - p.w_min) / p.nw : (p.w_max - p.w_min);
+    StackArgs a{};
+    a.n = p.n;
+    split(p.pixel_rad * p.pixel_rad, &a.dl2_hi, &a.dl2_lo);
+    split(p.w_min + 0.5 * dw, &a.wb_hi, &a.wb_lo);
+    split(dw, &a.dw_hi, &a.dw_lo);
+    a.flags = p.flags;
+    a.wcorr = h->cfg.Sw > 1 ? h->wcorr : nullptr;
+    a.wc_scale = h->wc_scale;
+    a.wait_ns = h->dbg_wait_ns;
+    a.skip_slot1 = h->dbg_skip_slot1;
+    return a;
+}
+
+void strip_free(rick_handle h)
+{
+    cudaFree(h->strips);
+    cudaFree(h->sargs.bits);
+    cudaFree(h->sargs.range);
+    cudaFree(h->sargs.tab.rho);
+    cudaFree(const_cast<float2*>(h->sargs.tw1));
+    h->strips = nullptr;
+    h->sargs = StripArgs{};
+}
+
+// Buffers and twiddles of the strip transform (rick_create); false where they
+// do not fit.
+bool strip_alloc(rick_handle h)
+{
+    const GridCfg& c = h->cfg;
+    const size_t pb = plane_bytes(&h->p);
+    const int n = h->p.n, r = n / 256, wpr = (c.ntu + 31) / 32;
+    size_t fr = 0, tot = 0;
+    const size_t bits = (size_t)c.nw * c.ntu * wpr * sizeof(uint32_t), rng = (size_t)c.nw * sizeof(int2);
+    const size_t t1 = 15 * (size_t)(n / 16), t2 = 15 * (size_t)r, tw = (t1 + t2) * sizeof(float2);
+    const size_t tab = (size_t)h->nchan * (n / 2 + 1) * (n / 2 + 16);  // entries of each screen table
+    const size_t tab_bytes = 3 * tab * sizeof(float2);
+    const size_t need = (size_t)h->G * pb + bits + rng + tw + tab_bytes;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || need + (64u << 20) > fr) return false;
+    std::vector<float2> w(t1 + t2);
+    for (int k = 1; k < 16; ++k) {
+        for (int j = 0; j < n / 16; ++j) {
+            const double a = 6.283185307179586476925 * (double)((int64_t)j * k % n) / (double)n;
+            w[(k - 1) * (n / 16) + j] = make_float2((float)std::cos(a), (float)std::sin(a));
+        }
+        for (int j = 0; j < r; ++j) {
+            const double a = 6.283185307179586476925 * (double)(j * k % (n / 16)) / (double)(n / 16);
+            w[t1 + (k - 1) * r + j] = make_float2((float)std::cos(a), (float)std::sin(a));
+        }
+    }
+    float2* dev_tw = nullptr;
+    bool ok = cudaMalloc((void**)&h->strips, (size_t)h->G * pb) == cudaSuccess &&
+              cudaMalloc((void**)&h->sargs.bits, bits) == cudaSuccess &&
+              cudaMalloc((void**)&h->sargs.range, rng) == cudaSuccess &&
+              cudaMalloc((void**)&h->sargs.tab.rho, tab_bytes) == cudaSuccess &&
+              cudaMalloc((void**)&dev_tw, tw) == cudaSuccess;
+    h->sargs.tw1 = dev_tw;
+    h->sargs.tw2 = dev_tw ? dev_tw + t1 : nullptr;
+    h->sargs.tab.kap = h->sargs.tab.rho + tab;
+    h->sargs.tab.fin = h->sargs.tab.kap + tab;
+    ok = ok && cudaMemcpy(dev_tw, w.data(), tw, cudaMemcpyHostToDevice) == cudaSuccess;
+    ok = ok && encode_rows_map(h->rowsmap, h->strips, n, h->G) == cudaSuccess;
+    h->sargs.map = h->rowsmap;
+    StackArgs a = stack_args(h);
+    if (h->batch) a.chan_screen = h->chan_scr;
+    h->screen_k0 = 0;
+    ok = ok && launch_screen(h->sargs, a, h->taper, true, h->nchan, nullptr) == cudaSuccess;
+    if (!ok) {
+        (void)cudaGetLastError();
+        strip_free(h);
+        return false;
+    }
+    h->sargs.wpr = wpr;
+    h->sargs.log2T = c.log2T;
+    h->bytes_held += need;
+    return true;
+}
+
+// The screen tables of a group whose first plane is k0.
+rick_status strip_screen(rick_handle h, const StackArgs& a, int k0)
+{
+    if (h->screen_k0 == k0) return RICK_OK;
+    StackArgs b = a;
+    b.k0 = k0;
+    RICK_CU(h, launch_screen(h->sargs, b, h->taper, false, 1, h->stream));
+    h->screen_k0 = k0;
+    count_launches(h, 1);
+    return RICK_OK;
+}
+
 // Grid planes [k0, k0 + nk) of every stored chunk into `planes`: the
 // handle's own buffer (its row order) or a caller's (natural rows).
 rick_status grid_pass(rick_handle h, int k0, int nk, bool shift, float2* planes, bool natural_rows = false)
@@ -348,18 +477,14 @@ rick_status grid_pass(rick_handle h, int k0, int nk, bool shift, float2* planes,
     const size_t nch = h->chunks.size();
     size_t c0 = 0;
     do {
-        ChunkList cl{};
-        cl.count = 0;
-        for (size_t q = c0; q < nch && cl.count < kMaxChunksPerPass; ++q, ++cl.count) {
-            cl.off[cl.count] = h->chunks[q].off;
-            cl.ent[cl.count] = h->chunks[q].ent;
-        }
+        const ChunkList cl = chunk_list(h, c0);
         // the heavy-tile list (used when the pass has one chunk) is sized
         // for that chunk's entry bound, stream-ordered from the pool
         const size_t words = cl.count == 1 ? heavy_words_for(h->chunks[c0].cap) : 4;
         uint32_t* heavy = nullptr;
         RICK_CU(h, cudaMallocFromPoolAsync((void**)&heavy, words * sizeof(uint32_t), h->pool, h->stream));
-        const cudaError_t e = launch_grid(cfg, cl, k0, nk, shift, c0 > 0, heavy, words, planes, h->stream);
+        const cudaError_t e = launch_grid(cfg, cl, k0, nk, shift, c0 > 0, heavy, words, planes, h->stream,
+                                          !natural_rows && skips_empty(h));
         cudaFreeAsync(heavy, h->stream);
         RICK_CU(h, e);
         count_launches(h, 2);
@@ -437,6 +562,9 @@ rick_status rick_workspace_size(const rick_params* p, int64_t max_vis, size_t* b
     b += (size_t)entries_bound(c, max_vis) * sizeof(float4);         // entries
     b += heavy_words_for(entries_bound(c, max_vis)) * sizeof(uint32_t);  // gridder's heavy-tile list
     if (p->flags & RICK_UNIFORM_WEIGHT) b += (size_t)c.n * c.n * sizeof(uint32_t);
+    if (want_strip(*p))  // the strip order's copy of a group, tile bits, row ranges, twiddles, screen
+        b += (size_t)G * plane_bytes(p) + (size_t)c.nw * (c.ntu * ((c.ntu + 31) / 32) + 2) * sizeof(uint32_t) +
+             ((size_t)15 * (c.n / 16 + c.n / 256) + 3 * (size_t)(c.n / 2 + 1) * (c.n / 2 + 16)) * sizeof(float2);
     b += plane_bytes(p);                                             // cuFFT work area (estimate)
     *bytes = b;
     return RICK_OK;
@@ -506,10 +634,24 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
     const GridCfg& c = h->cfg;
     const int64_t ntiles = (int64_t)c.nw * c.ntp;
     size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-        delete h;
-        return RICK_ERR_CUDA;
+    auto cleanup = [&](rick_status st) {
+        snprintf(g_create_error, sizeof(g_create_error), "%s",
+                 h->last_error[0] ? h->last_error : rick_status_string(st));
+        rick_destroy(h);
+        return st;
+    };
+    if (cudaMalloc(&h->taper, (size_t)c.n * sizeof(float)) != cudaSuccess) return cleanup(RICK_ERR_OOM);
+    if (launch_taper(c, h->kernel_param, h->taper, nullptr) != cudaSuccess) return cleanup(RICK_ERR_CUDA);
+    h->amp = 1.0;
+    if (p->flags & RICK_GRID_CORRECT) {
+        std::vector<float> tap(c.n);
+        if (cudaMemcpy(tap.data(), h->taper, sizeof(float) * c.n, cudaMemcpyDeviceToHost) != cudaSuccess)
+            return cleanup(RICK_ERR_CUDA);
+        double s2 = 0.0;
+        for (float x : tap) s2 += 1.0 / ((double)x * (double)x);
+        h->amp = s2 / c.n;
     }
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return cleanup(RICK_ERR_CUDA);
     // plane group: as requested, else as many planes as fit in 60 % of free memory;
     // in batched imaging a group holds whole channels
     const size_t pb = plane_bytes(p);
@@ -517,10 +659,10 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
     int G = p->plane_group ? p->plane_group : NW;
     if (G > NW) G = NW;
     if (!p->plane_group) {
-        // planes + cuFFT's work area: the 2D plan may need as much as the
-        // planes, the split transform's row plan far less
+        // planes + cuFFT's work area or the strip buffer: the 2D plan may need
+        // as much as the planes, the split transform's row plan far less
         int n1 = 0, n2 = 0;
-        const bool split = !h->batch && use_split(*p, &n1, &n2);
+        const bool split = !h->batch && use_split(*p, &n1, &n2) && !(want_strip(*p) && h->amp <= kStripAmp);
         const size_t fit = split ? (size_t)(0.7 * (double)fr) / (pb ? pb : 1)
                                  : (size_t)(0.6 * (double)fr) / (pb ? 2 * pb : 1);
         if ((size_t)G > fit) G = (int)(fit > 0 ? fit : 1);
@@ -532,17 +674,7 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
     h->G = G;
     size_t need = (size_t)G * pb + (G < NW ? pb : 0) + (size_t)ntiles * 4 + (size_t)c.n * 4 +
                   ((p->flags & RICK_UNIFORM_WEIGHT) ? (size_t)c.n * c.n * 4 : 0) + (64u << 20);
-    if (need > fr) {
-        delete h;
-        return RICK_ERR_OOM;
-    }
-    auto cleanup = [&](rick_status st) {
-        snprintf(g_create_error, sizeof(g_create_error), "%s",
-                 h->last_error[0] ? h->last_error : rick_status_string(st));
-        rick_destroy(h);
-        return st;
-    };
-    if (cudaMalloc(&h->taper, (size_t)c.n * sizeof(float)) != cudaSuccess) return cleanup(RICK_ERR_OOM);
+    if (need > fr) return cleanup(RICK_ERR_OOM);
     if (cudaMalloc(&h->planes, (size_t)G * pb) != cudaSuccess) return cleanup(RICK_ERR_OOM);
     if (G < NW && !h->batch && cudaMalloc(&h->acc, pb) != cudaSuccess) return cleanup(RICK_ERR_OOM);
     if (h->batch) {
@@ -606,7 +738,6 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
                     scan_block_sums_len(ntiles) * 4 + sizeof(Counters) +
                     ((p->flags & RICK_UNIFORM_WEIGHT) ? (size_t)c.n * c.n * 4 : 0);
     if (cudaMemset(h->ctr, 0, sizeof(Counters)) != cudaSuccess) return cleanup(RICK_ERR_CUDA);
-    if (launch_taper(c, h->kernel_param, h->taper, nullptr) != cudaSuccess) return cleanup(RICK_ERR_CUDA);
     if (c.Sw > 1) {
         // -(n - 1) over the image reaches its largest value at the corners
         const double half = 0.5 * p->n * p->pixel_rad, r2 = 2.0 * half * half;
@@ -658,8 +789,9 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
             for (int j = 0; j < kPolyTerms; ++j) h->cfg.coef[t][j] = (t < c.S) ? coef[t * kPolyTerms + j] : 0.0f;
         set_tap_sum(h->cfg);
     }
+    h->strip = want_strip(*p) && h->amp <= kStripAmp && strip_alloc(h);
     // the cuFFT plans this handle's transform path uses
-    {
+    if (!h->strip) {
         cufftHandle plan;
         int n1 = 0, n2 = 0;
         // batches take the split from n = 1024 on (one row plan, one
@@ -716,6 +848,7 @@ rick_status rick_destroy(rick_handle h)
     }
     cudaFree(h->taper);
     cudaFree(h->cf_tw);
+    strip_free(h);
     cudaFree(h->sw_dev);
     cudaFree(h->planes);
     cudaFree(h->acc);
@@ -856,24 +989,23 @@ rick_status rick_fft_and_stack(rick_handle h, float* image)
     if (h->batch) return fail(h, RICK_ERR_STATE, "batched handle: use rick_image_batch");
     if (!image) return fail(h, RICK_ERR_ARG, "image is NULL");
     const rick_params& p = h->p;
-    const double dw = (p.nw > 1) ? (p.w_max - p.w_min) / p.nw : (p.w_max - p.w_min);
-    StackArgs a{};
-    a.n = p.n;
-    split(p.pixel_rad * p.pixel_rad, &a.dl2_hi, &a.dl2_lo);
-    split(p.w_min + 0.5 * dw, &a.wb_hi, &a.wb_lo);
-    split(dw, &a.dw_hi, &a.dw_lo);
-    a.flags = p.flags;
-    a.wcorr = h->cfg.Sw > 1 ? h->wcorr : nullptr;
-    a.wc_scale = h->wc_scale;
-    a.wait_ns = h->dbg_wait_ns;
-    a.skip_slot1 = h->dbg_skip_slot1;
-    // the split (use_split): cuFFT transforms the rows, k_colfft the first
+    StackArgs a = stack_args(h);
+    // the strip transform (rick_strip.cu) where the handle has it; else the
+    // split (use_split): cuFFT transforms the rows, k_colfft the first
     // factor of the columns, k_colstack the last factor with the screen and
     // the stack (planes in b-major row order, GridCfg::row_perm); otherwise
     // cuFFT's 2D plan and k_stack
     int n1 = 0, n2 = 0;
     const bool split = use_split(p, &n1, &n2);
     const int lo = h->cfg.plane_lo, hi = h->cfg.plane_hi;
+    StripArgs sa = h->sargs;
+    if (h->strip) {  // the tiles and rows the transform works on
+        ChunkList cl = chunk_list(h, 0);
+        if (!skips_empty(h)) cl.count = -1;
+        PhaseScope fs(h, kPhasePrep);
+        RICK_CU(h, launch_occupancy(h->cfg, cl, 0, sa, h->stream));
+        count_launches(h, 1);
+    }
     for (int k0 = lo; k0 < hi; k0 += h->G) {
         const int nk = (hi - k0 < h->G) ? hi - k0 : h->G;
         rick_status s = grid_pass(h, k0, nk, true, h->planes);
@@ -883,7 +1015,17 @@ rick_status rick_fft_and_stack(rick_handle h, float* image)
         a.nk = nk;
         a.first = (k0 == lo);
         a.last = (k0 + nk >= hi);
-        if (split) {
+        if (h->strip) {
+            sa.k0 = k0;
+            {
+                PhaseScope fs(h, kPhaseFft);
+                RICK_CU(h, launch_rows(p.n, +1, sa, k0, nk, h->planes, h->strips, h->dbg_wait_ns, &h->ctr->err, h->stream));
+                count_launches(h, 1);
+            }
+            PhaseScope ss(h, kPhaseStack);
+            if ((s = strip_screen(h, a, k0))) return s;
+            RICK_CU(h, launch_colimage(sa, a, h->strips, h->acc, norm_sum(h), image, &h->ctr->err, h->stream));
+        } else if (split) {
             cufftHandle rows;
             if ((s = get_plan(h, nk, &rows, kPlanRows))) return s;
             if ((s = colfft_ready(h))) return s;
@@ -945,15 +1087,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
         return fail(h, RICK_ERR_OOM, "cudaMallocFromPoolAsync(perm): %s", cudaGetErrorString(e));
     }
     float2* grad = reinterpret_cast<float2*>(vis_grad);
-    const double dw = (p.nw > 1) ? (p.w_max - p.w_min) / p.nw : (p.w_max - p.w_min);
-    StackArgs a{};
-    a.n = p.n;
-    split(p.pixel_rad * p.pixel_rad, &a.dl2_hi, &a.dl2_lo);
-    split(p.w_min + 0.5 * dw, &a.wb_hi, &a.wb_lo);
-    split(dw, &a.dw_hi, &a.dw_lo);
-    a.flags = p.flags;
-    a.wcorr = h->cfg.Sw > 1 ? h->wcorr : nullptr;
-    a.wc_scale = h->wc_scale;
+    StackArgs a = stack_args(h);
     rick_status st = RICK_OK;
     e = cudaMemsetAsync(grad, 0, (size_t)nvis * sizeof(float2), h->stream);
     if (e == cudaSuccess)
@@ -963,17 +1097,42 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
     if (e == cudaSuccess) e = launch_primary_scatter(c, u, v, w, weights, nvis, h->cursor, perm, h->stream);
     if (e != cudaSuccess) st = fail(h, RICK_ERR_CUDA, "rick_degrid sort: %s", cudaGetErrorString(e));
     if (!st) count_launches(h, 5);
-    // the adjoint of rick_fft_and_stack's transform path: with the split,
+    // the adjoint of rick_fft_and_stack's transform path: with the strip
+    // transform k_colspread, then the row transforms of the needed tiles; with the split,
     // k_spreadcol writes the planes after the adjoint of the last column
     // factor, then k_colfft's forward first column factor and cuFFT's forward
     // rows; otherwise k_spread and cuFFT's forward 2D plan
     int n1 = 0, n2 = 0;
     const bool split = use_split(p, &n1, &n2);
     cufftComplex* planes = reinterpret_cast<cufftComplex*>(h->planes);
+    StripArgs sa = h->sargs;
+    if (!st && h->strip) {  // the tiles that the footprints touch
+        ChunkList cl{};
+        cl.off[0] = off;
+        cl.count = 1;
+        e = launch_occupancy(c, cl, c.Sw, sa, h->stream);
+        if (e != cudaSuccess) st = fail(h, RICK_ERR_CUDA, "k_occupancy: %s", cudaGetErrorString(e));
+        count_launches(h, 1);
+    }
     for (int k0 = c.plane_lo; !st && k0 < c.plane_hi; k0 += h->G) {
         const int nk = (c.plane_hi - k0 < h->G) ? c.plane_hi - k0 : h->G;
         a.k0 = k0;
         a.nk = nk;
+        if (h->strip) {
+            sa.k0 = k0;
+            if ((st = strip_screen(h, a, k0))) break;
+            e = launch_colspread(sa, a, image_grad, sum_w, h->strips, h->stream);
+            if (e == cudaSuccess)
+                e = launch_rows(p.n, -1, sa, k0, nk, h->planes, h->strips, h->dbg_wait_ns, &h->ctr->err, h->stream);
+            if (e == cudaSuccess)
+                e = launch_degrid_gather(c, perm, off, k0, nk, h->planes, u, v, w, weights, density, grad, h->stream);
+            if (e != cudaSuccess) {
+                st = fail(h, RICK_ERR_CUDA, "strip adjoint: %s", cudaGetErrorString(e));
+                break;
+            }
+            count_launches(h, 3);
+            continue;
+        }
         e = split ? launch_spreadcol(a, n1, n2, image_grad, h->taper, sum_w, h->planes, h->stream)
                   : launch_spread(a, image_grad, h->taper, sum_w, h->planes, h->stream);
         if (e != cudaSuccess) {
@@ -1262,6 +1421,13 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
         RICK_CU(h, launch_scatter(c, u, v, w, weights, vis2, m, nullptr, h->cursor, h->b_ent, h->ctr, h->chan_sw,
                                   h->stream));
         count_launches(h, 5);
+        if (h->strip) {
+            ChunkList cl{};
+            cl.off[0] = h->b_off;
+            cl.count = 1;
+            RICK_CU(h, launch_occupancy(c, cl, 0, h->sargs, h->stream));
+            count_launches(h, 1);
+        }
     }
     const size_t img_floats = (size_t)p.n * p.n * ((p.flags & RICK_REAL_IMAGE) ? 1 : 2);
     const size_t nn = (size_t)p.n * p.n;
@@ -1286,6 +1452,24 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
     // planes2) on stream st: cuFFT's rows, k_colfft, and per channel the
     // fused last column factor + w-screen + stack (k_colstack)
     auto split_group = [&](float2* buf, int b, int k0, int nk, cudaStream_t st) -> rick_status {
+        const int ch0 = k0 / c.nw_chan, nch = nk / c.nw_chan;
+        StackArgs a = chan_args(ch0);
+        a.plane0 = ch0 * c.nw_chan - k0;
+        a.chan_screen = h->chan_scr;
+        a.chan0 = ch0;
+        a.img_stride = (long long)img_floats;
+        if (h->strip) {
+            StripArgs sa = h->sargs;
+            sa.k0 = k0;
+            {
+                PhaseScope fs(h, kPhaseFft);
+                RICK_CU(h, launch_rows(p.n, +1, sa, k0, nk, buf, h->strips, h->dbg_wait_ns, &h->ctr->err, st));
+            }
+            PhaseScope ss(h, kPhaseStack);
+            RICK_CU(h, launch_colimage(sa, a, h->strips, nullptr, h->chan_sw, images, &h->ctr->err, st, nch));
+            count_launches(h, 2);
+            return RICK_OK;
+        }
         cufftHandle rows;
         rick_status s = get_plan(h, nk, &rows, kPlanRows);
         if (s) return s;
@@ -1305,12 +1489,6 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
         }
         // one launch over the group's channels (grid z = channel)
         PhaseScope ss(h, kPhaseStack);
-        const int ch0 = k0 / c.nw_chan, nch = nk / c.nw_chan;
-        StackArgs a = chan_args(ch0);
-        a.plane0 = ch0 * c.nw_chan - k0;
-        a.chan_screen = h->chan_scr;
-        a.chan0 = ch0;
-        a.img_stride = (long long)img_floats;
         RICK_CU(h, launch_colstack(b ? h->colmap2 : h->colmap, a, n1, n2, nullptr, h->taper, h->chan_sw, images,
                                    &h->ctr->err, st, nch));
         count_launches(h, 1);
@@ -1331,7 +1509,7 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
         cl.off[0] = h->b_off;
         cl.ent[0] = h->b_ent;
         cl.count = 1;
-        RICK_CU(h, launch_grid(c, cl, k0, nk, true, false, h->b_heavy, h->b_heavy_words, buf, h->stream));
+        RICK_CU(h, launch_grid(c, cl, k0, nk, true, false, h->b_heavy, h->b_heavy_words, buf, h->stream, h->strip));
         count_launches(h, 2);
         return RICK_OK;
     };
@@ -1352,7 +1530,7 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
             if (s) return s;
             RICK_CU(h, cudaEventRecord(h->ev_gridded[b], h->stream));
             RICK_CU(h, cudaStreamWaitEvent(h->fft_stream, h->ev_gridded[b], 0));
-            if (h->batch_split) {
+            if (h->batch_split || h->strip) {
                 if ((s = split_group(buf, b, k0, nk, h->fft_stream))) return s;
             } else {
                 cufftHandle plan;
@@ -1376,7 +1554,7 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
             rick_status s = grid_group(h->planes, k0, nk);
             if (s) return s;
         }
-        if (h->batch_split) {
+        if (h->batch_split || h->strip) {
             rick_status s = split_group(h->planes, 0, k0, nk, h->stream);
             if (s) return s;
             continue;
@@ -1457,7 +1635,7 @@ rick_status rick_image_batch(rick_handle h, const float* vis, const float* u, co
         // per plane group the two gridder kernels, then k_colfft and one
         // k_colstack over its channels (split) or one k_stack per channel
         const int groups = (c.nw + h->G - 1) / h->G;
-        count_launches(h, 5 + (h->batch_split ? 4 * groups : 2 * groups + h->nchan));
+        count_launches(h, h->strip ? 6 + 4 * groups : 5 + (h->batch_split ? 4 * groups : 2 * groups + h->nchan));
         return RICK_OK;
     }
     if (!use_graph) return batch_body(h, vis, u, v, w, weights, m, images);

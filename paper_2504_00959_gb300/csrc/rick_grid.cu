@@ -460,8 +460,8 @@ __device__ __forceinline__ bool list_heavy(const HeavyList& hl, uint32_t n, uint
 // Lane q < ch.count holds the range of list q for the tile.
 template <int S>
 __global__ void __launch_bounds__(256, S <= 8 ? 2 : 0) k_grid_tiles(GridCfg c, ChunkList ch, int k0, int64_t ntl,
-                                                                   int shift,
-                                                    int accumulate, float2* __restrict__ planes, HeavyList hl)
+                                                                   int shift, int accumulate, int skip_empty,
+                                                                   float2* __restrict__ planes, HeavyList hl)
 {
     extern __shared__ float4 smem4[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(256, S <= 8 ? 2 : 0) k_grid_tiles(GridCfg c, C
                 const TileGeom g = tile_geom(c, k0, tl + (int64_t)(k + q) * nwt);
                 float2* P0 = planes + (int64_t)g.kl * c.n * c.n;
                 if (cq == 0) {
-                    if (!accumulate) store_tile<true>(c, g, P0, nullptr, lane);
+                    if (!accumulate && !skip_empty) store_tile<true>(c, g, P0, nullptr, lane);
                     continue;
                 }
                 init_tile(c, g, P0, tile4, accumulate != 0, lane);
@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(256, S <= 8 ? 2 : 0) k_grid_tiles(GridCfg c, C
         // it; with no room left in the lists, grid it here (correct, slower)
         if (nent > heavy && ch.count == 1 && list_heavy(hl, nent, (uint32_t)tl, lane)) continue;
         if (nent == 0) {
-            if (!accumulate) store_tile<true>(c, g, P0, nullptr, lane);
+            if (!accumulate && !skip_empty) store_tile<true>(c, g, P0, nullptr, lane);
             continue;
         }
         init_tile(c, g, P0, tile4, accumulate != 0, lane);
@@ -885,7 +885,7 @@ cudaError_t grid_launch_info(int T, size_t tile_bytes, int hw, GridLaunchInfo& o
 
 template <int S>
 cudaError_t launch_grid_s(const GridCfg& c, const ChunkList& ch, int k0, int nk, bool shift, bool accumulate,
-                          float2* planes, uint32_t* heavy, size_t heavy_words, cudaStream_t s)
+                          bool skip_empty, float2* planes, uint32_t* heavy, size_t heavy_words, cudaStream_t s)
 {
     const int64_t ntl = (int64_t)nk * c.ntp;
     if (ntl <= 0) return cudaSuccess;
@@ -909,7 +909,7 @@ cudaError_t launch_grid_s(const GridCfg& c, const ChunkList& ch, int k0, int nk,
     if ((e = cudaMemsetAsync(heavy, 0, 4 * sizeof(uint32_t), s)) != cudaSuccess) return e;
     const unsigned tile_blocks = (unsigned)((nblocks + kTilesPerWarp - 1) / kTilesPerWarp);
     k_grid_tiles<S><<<tile_blocks, 32 * wl, tile_bytes * wl, s>>>(c, ch, k0, ntl, shift ? 1 : 0, accumulate ? 1 : 0,
-                                                                  planes, hl);
+                                                                  skip_empty ? 1 : 0, planes, hl);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // persistent: as many clusters as are co-resident
     cudaLaunchAttribute at[1];
@@ -935,12 +935,13 @@ size_t heavy_words_for(int64_t max_entries)
 }
 
 cudaError_t launch_grid(const GridCfg& c, const ChunkList& ch, int k0, int nk, bool shift_sign,
-                        bool accumulate, uint32_t* heavy, size_t heavy_words, float2* planes, cudaStream_t s)
+                        bool accumulate, uint32_t* heavy, size_t heavy_words, float2* planes, cudaStream_t s,
+                        bool skip_empty)
 {
     if (!heavy || heavy_words < 4) return cudaErrorInvalidValue;
     switch (c.S) {
 #define RICK_GRID_CASE(SS) \
-    case SS: return launch_grid_s<SS>(c, ch, k0, nk, shift_sign, accumulate, planes, heavy, heavy_words, s);
+    case SS: return launch_grid_s<SS>(c, ch, k0, nk, shift_sign, accumulate, skip_empty, planes, heavy, heavy_words, s);
         RICK_GRID_CASE(1) RICK_GRID_CASE(2) RICK_GRID_CASE(3) RICK_GRID_CASE(4)
         RICK_GRID_CASE(5) RICK_GRID_CASE(6) RICK_GRID_CASE(7) RICK_GRID_CASE(8)
         RICK_GRID_CASE(9) RICK_GRID_CASE(10) RICK_GRID_CASE(11) RICK_GRID_CASE(12)

@@ -254,8 +254,11 @@ cudaError_t launch_scatter(const GridCfg& c, const float* u, const float* v, con
 // tiles (four counters, then one word per tile; a tile that does not fit is
 // gridded by one warp, correct but slower).  heavy_words_for() gives the size
 // that never overflows for a pass over at most max_entries entries.
+// skip_empty: tiles without entries are left unwritten (the reader knows them,
+// k_occupancy) instead of being written as zeros.
 cudaError_t launch_grid(const GridCfg& c, const ChunkList& chunks, int k0, int nk, bool shift_sign,
-                        bool accumulate, uint32_t* heavy, size_t heavy_words, float2* planes, cudaStream_t s);
+                        bool accumulate, uint32_t* heavy, size_t heavy_words, float2* planes, cudaStream_t s,
+                        bool skip_empty = false);
 size_t heavy_words_for(int64_t max_entries);
 cudaError_t launch_taper(const GridCfg& c, double kernel_param, float* taper, cudaStream_t s);
 // The Fourier transform of the w-kernel at xi_j = xi_max j / (len - 1), j < len.
@@ -331,6 +334,47 @@ cudaError_t launch_colfft(const void* map, const float2* tw, float2* planes, int
                           unsigned long long wait_ns, unsigned long long* err, cudaStream_t s);
 cudaError_t launch_spreadcol(const StackArgs& a, int n1, int n2, const void* rimg, const float* taper,
                              const double* sum_w, float2* planes, cudaStream_t s);
+
+// ---- the two-pass transform of n = 1024, 2048, 4096 (rick_strip.cu)
+// The w-screen of the pixels (k_screen): [nchan][n / 2 + 1][n / 2 + 16] each.
+struct ScreenTab {
+    float2* rho;  // rotation between planes
+    float2* kap;  // its correction over 32 planes
+    float2* fin;  // screen of the group's first plane times the finalisation
+};
+// What the kernels share: tile bits (wpr words per tile row) and non-empty
+// tile-row ranges of all planes of the handle (k_occupancy), the first plane
+// of the group that is in the strip buffer, and the twiddles w_n^(j k1)
+// ([15][n / 16], k1 = 1 .. 15) and w_(n/16)^(t2 k2) ([15][n / 256]).
+struct StripArgs {
+    uint32_t* bits;
+    int2* range;
+    int wpr, log2T, k0;
+    const float2* tw1;
+    const float2* tw2;
+    ScreenTab tab;
+    const void* map;  // tensor map of the strip buffer (encode_rows_map)
+};
+cudaError_t encode_rows_map(void* map, const float2* strips, int n, int planes);
+bool strip_shape(int n);
+// reach 0: tiles with entries in any of the lists (list count -1: all tiles);
+// reach > 0: tiles that the footprints of an adjoint sort (one list) touch,
+// w-footprints of `reach` planes
+cudaError_t launch_occupancy(const GridCfg& c, const ChunkList& ch, int reach, const StripArgs& s, cudaStream_t st);
+// the screen tables of nchan channels (chan_screen) or of the single image,
+// fin for the first plane a.k0; rho and kap only when with_rho
+cudaError_t launch_screen(const StripArgs& s, const StackArgs& a, const float* taper, bool with_rho, int nchan,
+                          cudaStream_t st);
+// dir +1: natural rows of planes [k0, k0 + nk) -> strips; -1: strips -> the needed tiles of the natural rows
+cudaError_t launch_rows(int n, int dir, const StripArgs& s, int k0, int nk, float2* planes, float2* strips,
+                        unsigned long long wait_ns, unsigned long long* err, cudaStream_t st);
+// sum_w and image: of the single image, or of channel 0 of a batch (a.chan0 + z is this launch's channel z)
+cudaError_t launch_colimage(const StripArgs& s, const StackArgs& a, const float2* strips, float2* acc,
+                            const double* sum_w, void* image, unsigned long long* err, cudaStream_t st,
+                            int nchan = 1);
+cudaError_t launch_colspread(const StripArgs& s, const StackArgs& a, const void* rimg, const double* sum_w,
+                             float2* strips, cudaStream_t st);
+
 cudaError_t launch_stack(const StackArgs& a, const float2* planes, float2* acc, const float* taper,
                          const double* sum_w, void* image, cudaStream_t s);
 
@@ -400,6 +444,14 @@ struct rick_imager {
     bool batch_split;
     alignas(64) unsigned char colmap2[128];
     alignas(64) unsigned char cfmap2[128];
+    // the two-pass transform (rick_strip.cu): the strip buffer of a group, the
+    // tile bits and row ranges of every plane, and the twiddles
+    double amp;                      // what the grid correction does to rounding: mean 1 / taper^2 (1 without)
+    bool strip;
+    float2* strips;                  // [G][n / 2][n] pairs of columns
+    rick::StripArgs sargs;
+    int screen_k0;                   // the first plane sargs.tab.fin is for
+    alignas(64) unsigned char rowsmap[128];  // tensor map of `strips` for k_rows
     float2* cf_tw;                   // [n / 16] exp(+2 pi i j / (n / 16)) for k_colfft
     struct Chunk {
         uint32_t* off;

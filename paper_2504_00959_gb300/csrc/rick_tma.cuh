@@ -82,6 +82,22 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// one 2D tensor copy (TMA) of the box in shared memory to (x, y), in the
+// thread's current bulk group
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int xc, int yc, uint32_t src)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(xc), "r"(yc), "r"(src)
+                 : "memory");
+}
+
+// wait until the thread's bulk stores so far have read their shared memory
+__device__ __forceinline__ void bulk_store_drain()
+{
+    asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+
 // one bulk copy (TMA, untiled) of `bytes` bytes (a multiple of 16; both
 // addresses 16-byte aligned) from global memory into shared memory,
 // completing its bytes on the mbarrier
