@@ -215,6 +215,10 @@ bool want_strip(const rick_params& p) { return strip_shape(p.n) && !(p.flags & R
 // well above its rounding whatever the transform; beyond, a handle keeps the
 // transform that it always had, so that its images stay the same.
 constexpr double kStripAmp = 300.0;
+// The adjoint's footprints, of planes that hold the corrected image, cancel by
+// the same factors: where they cancel by more than binary32 holds, the gather
+// keeps its order of summation too.
+constexpr double kGatherAmp = 1e5;
 
 rick_status get_plan(rick_handle h, int batch, cufftHandle* out, int kind = kPlan2D)
 {
@@ -1073,15 +1077,18 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
     const rick_params& p = h->p;
     const int64_t ntiles = (int64_t)c.nw * c.ntp;
     const size_t off_bytes = (size_t)(ntiles + 1) * sizeof(uint32_t);
-    const size_t perm_bytes = (size_t)nvis * sizeof(uint32_t);
     size_t fr = 0, tot = 0;
     RICK_CU(h, cudaMemGetInfo(&fr, &tot));
+    // the sorted measurements where they fit, else their indices
+    const bool by_rows = !(h->amp <= kGatherAmp);
+    const bool with_entries = !by_rows && off_bytes + primary_list_bytes(nvis, true) + (64u << 20) <= fr;
+    const size_t perm_bytes = primary_list_bytes(nvis, with_entries);
     if (off_bytes + perm_bytes + (64u << 20) > fr) return fail(h, RICK_ERR_OOM, "degrid scratch does not fit");
     PhaseScope scope(h, kPhaseDegrid);
     uint32_t* off = nullptr;
-    uint32_t* perm = nullptr;
+    void* perm = nullptr;
     RICK_CU(h, cudaMallocFromPoolAsync((void**)&off, off_bytes, h->pool, h->stream));
-    cudaError_t e = cudaMallocFromPoolAsync((void**)&perm, perm_bytes, h->pool, h->stream);
+    cudaError_t e = cudaMallocFromPoolAsync(&perm, perm_bytes, h->pool, h->stream);
     if (e != cudaSuccess) {
         cudaFreeAsync(off, h->stream);
         return fail(h, RICK_ERR_OOM, "cudaMallocFromPoolAsync(perm): %s", cudaGetErrorString(e));
@@ -1094,7 +1101,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
         e = cudaMemsetAsync(h->cursor, 0, (size_t)ntiles * c.cstride * sizeof(uint32_t), h->stream);
     if (e == cudaSuccess) e = launch_primary_count(c, u, v, w, weights, nvis, h->cursor, h->stream);
     if (e == cudaSuccess) e = launch_scan(h->cursor, ntiles, c.cstride, off, h->cursor, h->block_sums, h->stream);
-    if (e == cudaSuccess) e = launch_primary_scatter(c, u, v, w, weights, nvis, h->cursor, perm, h->stream);
+    if (e == cudaSuccess) e = launch_primary_scatter(c, u, v, w, weights, nvis, density, h->cursor, perm, with_entries, h->stream);
     if (e != cudaSuccess) st = fail(h, RICK_ERR_CUDA, "rick_degrid sort: %s", cudaGetErrorString(e));
     if (!st) count_launches(h, 5);
     // the adjoint of rick_fft_and_stack's transform path: with the strip
@@ -1125,7 +1132,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
             if (e == cudaSuccess)
                 e = launch_rows(p.n, -1, sa, k0, nk, h->planes, h->strips, h->dbg_wait_ns, &h->ctr->err, h->stream);
             if (e == cudaSuccess)
-                e = launch_degrid_gather(c, perm, off, k0, nk, h->planes, u, v, w, weights, density, grad, h->stream);
+                e = launch_degrid_gather(c, perm, with_entries, by_rows, nvis, off, k0, nk, h->planes, u, v, w, weights, density, grad, h->stream);
             if (e != cudaSuccess) {
                 st = fail(h, RICK_ERR_CUDA, "strip adjoint: %s", cudaGetErrorString(e));
                 break;
@@ -1160,7 +1167,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
             st = fail(h, RICK_ERR_CUFFT, "cufftExecC2C(FORWARD): error %d", (int)r);
             break;
         }
-        e = launch_degrid_gather(c, perm, off, k0, nk, h->planes, u, v, w, weights, density, grad, h->stream);
+        e = launch_degrid_gather(c, perm, with_entries, by_rows, nvis, off, k0, nk, h->planes, u, v, w, weights, density, grad, h->stream);
         if (e != cudaSuccess) {
             st = fail(h, RICK_ERR_CUDA, "k_degrid_gather: %s", cudaGetErrorString(e));
             break;

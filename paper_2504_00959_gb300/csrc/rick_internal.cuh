@@ -384,11 +384,16 @@ cudaError_t launch_spread(const StackArgs& a, const void* rimg, const float* tap
 // (no duplication), then gather each measurement's footprint of a plane group
 cudaError_t launch_primary_count(const GridCfg& c, const float* u, const float* v, const float* w,
                                  const float* wt, int64_t m, uint32_t* counts, cudaStream_t s);
+// list: scratch of primary_list_bytes(m, with_entries), the sorted measurements
+// themselves or (less scratch) their indices
+size_t primary_list_bytes(int64_t m, bool with_entries);
 cudaError_t launch_primary_scatter(const GridCfg& c, const float* u, const float* v, const float* w,
-                                   const float* wt, int64_t m, uint32_t* cursor, uint32_t* perm,
-                                   cudaStream_t s);
-cudaError_t launch_degrid_gather(const GridCfg& c, const uint32_t* perm, const uint32_t* offsets, int k0, int nk,
-                                 const float2* planes, const float* u, const float* v, const float* w,
+                                   const float* wt, int64_t m, const uint32_t* density, uint32_t* cursor,
+                                   void* list, bool with_entries, cudaStream_t s);
+// by_rows: one thread per measurement, the footprint summed row by row (a list
+// of indices)
+cudaError_t launch_degrid_gather(const GridCfg& c, void* list, bool with_entries, bool by_rows, int64_t m,
+                                 const uint32_t* offsets, int k0, int nk, const float2* planes, const float* u, const float* v, const float* w,
                                  const float* wt, const uint32_t* density, float2* grad, cudaStream_t s);
 
 size_t scan_block_sums_len(int64_t len);
