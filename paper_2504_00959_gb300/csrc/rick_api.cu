@@ -1023,7 +1023,7 @@ rick_status rick_fft_and_stack(rick_handle h, float* image)
             sa.k0 = k0;
             {
                 PhaseScope fs(h, kPhaseFft);
-                RICK_CU(h, launch_rows(p.n, +1, sa, k0, nk, h->planes, h->strips, h->dbg_wait_ns, &h->ctr->err, h->stream));
+                RICK_CU(h, launch_rows(p.n, +1, sa, k0, nk, h->planes, h->dbg_wait_ns, &h->ctr->err, h->stream));
                 count_launches(h, 1);
             }
             PhaseScope ss(h, kPhaseStack);
@@ -1130,7 +1130,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
             if ((st = strip_screen(h, a, k0))) break;
             e = launch_colspread(sa, a, image_grad, sum_w, h->strips, h->stream);
             if (e == cudaSuccess)
-                e = launch_rows(p.n, -1, sa, k0, nk, h->planes, h->strips, h->dbg_wait_ns, &h->ctr->err, h->stream);
+                e = launch_rows(p.n, -1, sa, k0, nk, h->planes, h->dbg_wait_ns, &h->ctr->err, h->stream);
             if (e == cudaSuccess)
                 e = launch_degrid_gather(c, perm, with_entries, by_rows, nvis, off, k0, nk, h->planes, u, v, w, weights, density, grad, h->stream);
             if (e != cudaSuccess) {
@@ -1470,7 +1470,7 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
             sa.k0 = k0;
             {
                 PhaseScope fs(h, kPhaseFft);
-                RICK_CU(h, launch_rows(p.n, +1, sa, k0, nk, buf, h->strips, h->dbg_wait_ns, &h->ctr->err, st));
+                RICK_CU(h, launch_rows(p.n, +1, sa, k0, nk, buf, h->dbg_wait_ns, &h->ctr->err, st));
             }
             PhaseScope ss(h, kPhaseStack);
             RICK_CU(h, launch_colimage(sa, a, h->strips, nullptr, h->chan_sw, images, &h->ctr->err, st, nch));

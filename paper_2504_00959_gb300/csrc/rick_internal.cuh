@@ -366,7 +366,7 @@ cudaError_t launch_occupancy(const GridCfg& c, const ChunkList& ch, int reach, c
 cudaError_t launch_screen(const StripArgs& s, const StackArgs& a, const float* taper, bool with_rho, int nchan,
                           cudaStream_t st);
 // dir +1: natural rows of planes [k0, k0 + nk) -> strips; -1: strips -> the needed tiles of the natural rows
-cudaError_t launch_rows(int n, int dir, const StripArgs& s, int k0, int nk, float2* planes, float2* strips,
+cudaError_t launch_rows(int n, int dir, const StripArgs& s, int k0, int nk, float2* planes,
                         unsigned long long wait_ns, unsigned long long* err, cudaStream_t st);
 // sum_w and image: of the single image, or of channel 0 of a batch (a.chan0 + z is this launch's channel z)
 cudaError_t launch_colimage(const StripArgs& s, const StackArgs& a, const float2* strips, float2* acc,

@@ -145,7 +145,6 @@ template <int N>
 struct RowShape {
     static constexpr int r = N / 256, kPer = N / 16, R = 8192 / N, P = kPer + 1;
     static constexpr int kRowPitch = N + 16 + 16 / R;
-    static constexpr bool kImage = R < 4;  // strips written by TMA from a shared-memory image
 };
 
 // The row transforms of R rows at a time (64 KB of shared memory, two blocks
@@ -154,10 +153,10 @@ struct RowShape {
 // strips' side moves by TMA, from and to a [strip][row][2] image of the rows
 // in shared memory (map: the strip buffer as [strips][2 n] values, boxes of 2 R
 // values x 256 strips): each 16 R-byte piece would cost a store or load
-// instruction of the SM one pass of its own (n = 4096, pieces of 32 bytes:
-// 1.24 -> 1.10 ms for 32 planes; from 64 bytes on, n <= 2048, direct stores are
-// as fast and the image is left out).  The next rows' loads are in flight while
-// the image is written out (+1) or the last pass runs (-1).  A
+// instruction of the SM one pass of its own (direct stores: 1.24 instead of
+// 1.09 ms for 32 planes of 4096^2, 1.72 instead of 1.13 for 128 of 2048^2).  The
+// next rows' loads are in flight while the image is written out (+1) or the
+// last pass runs (-1).  A
 // warp's 32 lanes are 16 adjacent columns of 2 rows (natural rows: 128
 // contiguous bytes per half warp), or pairs of adjacent columns of all R rows
 // (16 R contiguous bytes of the image each).
@@ -192,8 +191,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const __grid_constant__
                                                          const float2* __restrict__ tw2,
                                                          const uint32_t* __restrict__ bits,
                                                          const int2* __restrict__ range, int k0,
-                                                         float2* __restrict__ planes, float2* __restrict__ strips,
-                                                         unsigned long long wait_ns,
+                                                         float2* __restrict__ planes, unsigned long long wait_ns,
                                                          unsigned long long* __restrict__ err)
 {
     using Sh = RowShape<N>;
@@ -339,7 +337,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const __grid_constant__
 #pragma unroll
             for (int o = 0; o < 16; ++o) x[o] = lds_c(blk + (g + r * (o / r)) * r + o % r);
         }
-        if (DIR < 0 || Sh::kImage) __syncthreads();  // the rows are read: their place takes an image
+        __syncthreads();  // the rows are read: their place takes an image
         if (DIR < 0 && t == 0 && v0 + stride < v1) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             fetch(v0 + stride);
@@ -355,10 +353,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const __grid_constant__
 #pragma unroll
             for (int k3 = 0; k3 < r; ++k3) {
                 const int col = k1 + 16 * (g + r * i) + 256 * k3;
-                if (DIR > 0 && Sh::kImage) {
+                if (DIR > 0) {
                     sts_c(sm + (col >> 1) * (2 * R) + 2 * row + (col & 1), y[k3]);
-                } else if (DIR > 0) {
-                    sts_c(strips + ((size_t)plane * (N / 2) + (col >> 1)) * (2 * N) + 2 * (v0 + row) + (col & 1), y[k3]);
                 } else {
                     if (need.at(16 * r * i + 256 * k3)) sts_c(nat + (size_t)(v0 + row) * N + col, y[k3]);
                 }
@@ -366,14 +362,12 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const __grid_constant__
         }
         if (DIR > 0) {
             if (v0 + stride < v1) load(v0 + stride);
-            if (Sh::kImage) {
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncthreads();
-                if (t == 0) {
-                    for (int q = 0; q < N / 2; q += kRowBox)
-                        tma_store_2d(&map, 2 * v0, plane * (N / 2) + q, smem_u32(sm + q * 2 * R));
-                    bulk_store_drain();  // the image is read until here
-                }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+            if (t == 0) {
+                for (int q = 0; q < N / 2; q += kRowBox)
+                    tma_store_2d(&map, 2 * v0, plane * (N / 2) + q, smem_u32(sm + q * 2 * R));
+                bulk_store_drain();  // the image is read until here
             }
             __syncthreads();
         }
@@ -875,29 +869,29 @@ cudaError_t opt_in(K kernel, size_t bytes, bool (&done)[64])
 }
 
 template <int N, int DIR, int LOG2T>
-cudaError_t launch_rows_n(const StripArgs& s, int k0, int nk, float2* planes, float2* strips, unsigned long long wait_ns,
+cudaError_t launch_rows_n(const StripArgs& s, int k0, int nk, float2* planes, unsigned long long wait_ns,
                           unsigned long long* err, cudaStream_t st)
 {
     static bool done[64] = {};
     const cudaError_t e = opt_in(k_rows<N, DIR, LOG2T>, rows_smem<N>(), done);
     if (e != cudaSuccess) return e;
-    // two blocks per SM and plane (a plane at a time): several row groups each at n = 4096
+    // two blocks per SM and plane (a plane at a time); n = 4096 gives each several row groups
     const int groups = N / RowShape<N>::R, want = 2 * sm_count_strip();
     const dim3 grid((unsigned)std::min(groups, want), (unsigned)nk);
     k_rows<N, DIR, LOG2T><<<grid, kRowThreads, rows_smem<N>(), st>>>(*reinterpret_cast<const CUtensorMap*>(s.map), s.tw1,
-                                                                    s.tw2, s.bits, s.range, k0, planes, strips, wait_ns, err);
+                                                                    s.tw2, s.bits, s.range, k0, planes, wait_ns, err);
     return cudaGetLastError();
 }
 
 template <int N>
-cudaError_t launch_rows_t(int dir, const StripArgs& s, int k0, int nk, float2* planes, float2* strips,
+cudaError_t launch_rows_t(int dir, const StripArgs& s, int k0, int nk, float2* planes,
                           unsigned long long wait_ns, unsigned long long* err, cudaStream_t st)
 {
     switch (s.log2T) {
 #define RICK_ROWS_CASE(L)                                                               \
     case L:                                                                             \
-        return dir > 0 ? launch_rows_n<N, 1, L>(s, k0, nk, planes, strips, wait_ns, err, st) \
-                       : launch_rows_n<N, -1, L>(s, k0, nk, planes, strips, wait_ns, err, st);
+        return dir > 0 ? launch_rows_n<N, 1, L>(s, k0, nk, planes, wait_ns, err, st) \
+                       : launch_rows_n<N, -1, L>(s, k0, nk, planes, wait_ns, err, st);
         RICK_ROWS_CASE(4)
         RICK_ROWS_CASE(5)
         RICK_ROWS_CASE(6)
@@ -967,15 +961,15 @@ cudaError_t launch_occupancy(const GridCfg& c, const ChunkList& ch, int reach, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_rows(int n, int dir, const StripArgs& s, int k0, int nk, float2* planes, float2* strips,
+cudaError_t launch_rows(int n, int dir, const StripArgs& s, int k0, int nk, float2* planes,
                         unsigned long long wait_ns, unsigned long long* err, cudaStream_t st)
 {
     if (nk <= 0) return cudaSuccess;
     if (nk > 65535) return cudaErrorInvalidValue;
     switch (n) {
-        case 1024: return launch_rows_t<1024>(dir, s, k0, nk, planes, strips, wait_ns, err, st);
-        case 2048: return launch_rows_t<2048>(dir, s, k0, nk, planes, strips, wait_ns, err, st);
-        case 4096: return launch_rows_t<4096>(dir, s, k0, nk, planes, strips, wait_ns, err, st);
+        case 1024: return launch_rows_t<1024>(dir, s, k0, nk, planes, wait_ns, err, st);
+        case 2048: return launch_rows_t<2048>(dir, s, k0, nk, planes, wait_ns, err, st);
+        case 4096: return launch_rows_t<4096>(dir, s, k0, nk, planes, wait_ns, err, st);
         default: return cudaErrorInvalidValue;
     }
 }
