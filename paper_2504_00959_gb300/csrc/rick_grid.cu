@@ -44,7 +44,13 @@ namespace {
 constexpr uint32_t kHeavyMin = 64;
 constexpr uint32_t kHeavyMax = 768;
 constexpr uint32_t kHeavyDiv = 16384;
+// Tiles a warp of k_grid_tiles takes: as many as leave every SM kTileWarps
+// warps, between one and kTilesPerWarp.  A run of tiles shares staging rounds
+// and hides their list reads, but with eight each the 4096 tiles of 16 planes of
+// 512^2 made 128 blocks of four warps, less than one per SM (gridding 163 -> 139
+// us with one each; 16 planes of 1024^2 137 -> 128, 12 of 1000^2 100 -> 92).
 constexpr int kTilesPerWarp = 8;
+constexpr int kTileWarps = 32;
 
 int sm_count_grid()
 {
@@ -453,21 +459,21 @@ __device__ __forceinline__ bool list_heavy(const HeavyList& hl, uint32_t n, uint
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-// Each CTA of W warps takes kTilesPerWarp * W consecutive tiles of the pass,
+// Each CTA of W warps takes tpw * W consecutive tiles of the pass,
 // warp w the tiles w, w + W, ... of them (neighbours, so similar loads), and
 // loads the next tile's list ranges while it grids the current one; the
 // hardware hands CTAs out dynamically, which balances the uneven tiles.
 // Lane q < ch.count holds the range of list q for the tile.
 template <int S>
 __global__ void __launch_bounds__(256, S <= 8 ? 2 : 0) k_grid_tiles(GridCfg c, ChunkList ch, int k0, int64_t ntl,
-                                                                   int shift, int accumulate, int skip_empty,
+                                                                   int shift, int accumulate, int skip_empty, int tpw,
                                                                    float2* __restrict__ planes, HeavyList hl)
 {
     extern __shared__ float4 smem4[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t nwt = blockDim.x >> 5;
-    const int64_t first = (int64_t)blockIdx.x * nwt * kTilesPerWarp;
-    const int64_t last = min(ntl, first + nwt * kTilesPerWarp);
+    const int64_t first = (int64_t)blockIdx.x * nwt * tpw;
+    const int64_t last = min(ntl, first + nwt * tpw);
     int64_t tl = first + wid;
     if (tl >= last) return;
     const uint32_t heavy = heavy_threshold(c, ch, k0, ntl);
@@ -478,7 +484,7 @@ __global__ void __launch_bounds__(256, S <= 8 ? 2 : 0) k_grid_tiles(GridCfg c, C
     ls.init(lane, pair_pitch(c.T));
 
     if constexpr (S <= 8) if (ch.count == 1) {
-        // One list: the warp's tiles tl + k nwt (k < kTilesPerWarp), lane k
+        // One list: the warp's tiles tl + k nwt (k < tpw), lane k
         // holding tile k's range.  Consecutive tiles with at most 32 entries
         // in all share one staging round (the taps of a light tile's few
         // entries would otherwise cost a whole round of polynomial
@@ -489,12 +495,12 @@ __global__ void __launch_bounds__(256, S <= 8 ? 2 : 0) k_grid_tiles(GridCfg c, C
         const uint32_t full = 0xffffffffu;
         const int64_t tk = tl + (int64_t)lane * nwt;
         uint32_t rb = 0, rn = 0;
-        if (lane < kTilesPerWarp && tk < last) {
+        if (lane < tpw && tk < last) {
             const int64_t tg = (int64_t)k0 * c.ntp + tk;
             rb = __ldg(ch.off[0] + tg);
             rn = __ldg(ch.off[0] + tg + 1) - rb;
         }
-        const int ntw = (int)min((int64_t)kTilesPerWarp, (last - tl + nwt - 1) / nwt);
+        const int ntw = (int)min((int64_t)tpw, (last - tl + nwt - 1) / nwt);
         const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(tile4);
         for (int k = 0; k < ntw;) {
             const uint32_t nk = __shfl_sync(full, rn, k);
@@ -907,9 +913,11 @@ cudaError_t launch_grid_s(const GridCfg& c, const ChunkList& ch, int k0, int nk,
     cudaError_t e = grid_launch_info<S>(c.T, tile_bytes, hw, info);
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(heavy, 0, 4 * sizeof(uint32_t), s)) != cudaSuccess) return e;
-    const unsigned tile_blocks = (unsigned)((nblocks + kTilesPerWarp - 1) / kTilesPerWarp);
+    const int64_t fit = ntl / ((int64_t)sm_count_grid() * kTileWarps);
+    const int tpw = (int)std::min<int64_t>(std::max<int64_t>(fit, 1), kTilesPerWarp);
+    const unsigned tile_blocks = (unsigned)((nblocks + tpw - 1) / tpw);
     k_grid_tiles<S><<<tile_blocks, 32 * wl, tile_bytes * wl, s>>>(c, ch, k0, ntl, shift ? 1 : 0, accumulate ? 1 : 0,
-                                                                  skip_empty ? 1 : 0, planes, hl);
+                                                                  skip_empty ? 1 : 0, tpw, planes, hl);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // persistent: as many clusters as are co-resident
     cudaLaunchAttribute at[1];
