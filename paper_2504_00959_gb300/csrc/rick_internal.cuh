@@ -375,8 +375,9 @@ cudaError_t launch_colimage(const StripArgs& s, const StackArgs& a, const float2
 cudaError_t launch_colspread(const StripArgs& s, const StackArgs& a, const void* rimg, const double* sum_w,
                              float2* strips, cudaStream_t st);
 
+// nchan > 1: channels a.chan0 .. of a batch in one launch (as launch_colstack)
 cudaError_t launch_stack(const StackArgs& a, const float2* planes, float2* acc, const float* taper,
-                         const double* sum_w, void* image, cudaStream_t s);
+                         const double* sum_w, void* image, cudaStream_t s, int nchan = 1);
 
 cudaError_t launch_spread(const StackArgs& a, const void* rimg, const float* taper, const double* sum_w,
                           float2* planes, cudaStream_t s);

@@ -23,11 +23,25 @@ namespace {
 constexpr int kStackThreads = 256;
 constexpr int kResync = 8;
 
-__global__ void __launch_bounds__(kStackThreads) k_stack(StackArgs a, const float2* __restrict__ planes,
+// grid y: the channel of a batch (chan_screen: its w-screen constants; its nk
+// planes, weight sum and image follow the ones before), or one image.
+__global__ void __launch_bounds__(kStackThreads) k_stack(StackArgs a_in, const float2* __restrict__ planes,
                                                          float2* __restrict__ acc,
                                                          const float* __restrict__ taper,
                                                          const double* __restrict__ sum_w, void* image)
 {
+    StackArgs a = a_in;
+    if (a_in.chan_screen) {
+        const int ch = a_in.chan0 + (int)blockIdx.y;
+        const float4 cs = __ldg(a_in.chan_screen + ch);
+        a.wb_hi = cs.x;
+        a.wb_lo = cs.y;
+        a.dw_hi = cs.z;
+        a.dw_lo = cs.w;
+        planes += (size_t)blockIdx.y * a.nk * a.n * a.n;
+        sum_w += ch;
+        image = reinterpret_cast<float*>(image) + (size_t)ch * a_in.img_stride;
+    }
     const int halfn = a.n >> 1;
     const int64_t idx = blockIdx.x * (int64_t)kStackThreads + threadIdx.x;
     if (idx >= (int64_t)a.n * halfn) return;
@@ -574,12 +588,13 @@ cudaError_t launch_spread(const StackArgs& a, const void* rimg, const float* tap
 }
 
 cudaError_t launch_stack(const StackArgs& a, const float2* planes, float2* acc, const float* taper,
-                         const double* sum_w, void* image, cudaStream_t s)
+                         const double* sum_w, void* image, cudaStream_t s, int nchan)
 {
+    if (nchan < 1 || nchan > 65535 || (nchan > 1 && !a.chan_screen)) return cudaErrorInvalidValue;
     const int64_t threads = (int64_t)a.n * (a.n / 2);
     const int64_t blocks = (threads + kStackThreads - 1) / kStackThreads;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    k_stack<<<(unsigned)blocks, kStackThreads, 0, s>>>(a, planes, acc, taper, sum_w, image);
+    k_stack<<<dim3((unsigned)blocks, (unsigned)nchan), kStackThreads, 0, s>>>(a, planes, acc, taper, sum_w, image);
     return cudaGetLastError();
 }
 
