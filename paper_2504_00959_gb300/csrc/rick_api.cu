@@ -215,6 +215,13 @@ bool want_strip(const rick_params& p) { return strip_shape(p.n) && !(p.flags & R
 // well above its rounding whatever the transform; beyond, a handle keeps the
 // transform that it always had, so that its images stay the same.
 constexpr double kStripAmp = 300.0;
+// The split transform's rows of n = 8192 and 16384 over what is not empty
+// (rick_longrow.cu) round differently in one factor of three only: up to the
+// Kaiser-Bessel kernel of support 8.  16384^2 x 16 planes x 2.5e7 measurements
+// 47.5 -> 41.4 ms (gridding 6.8 -> 4.9, rows 18.3 -> 13.6), 8192^2 x 4 x 3e4 2.76
+// -> 2.40 ms.
+constexpr double kLongAmp = 600.0;
+bool want_longrows(const rick_params& p) { return longrow_shape(p.n) && !(p.flags & RICK_FFT_2D); }
 // The adjoint's footprints, of planes that hold the corrected image, cancel by
 // the same factors: where they cancel by more than binary32 holds, the gather
 // keeps its order of summation too.
@@ -362,10 +369,10 @@ rick_status colfft_ready(rick_handle h)
     return RICK_OK;
 }
 
-// The tiles the strip transform reads and writes: those with entries in the
+// The tiles the strip transform and the sparse rows read and write: those with entries in the
 // stored chunks (all of them when the chunks take more than one pass, which
 // accumulates onto every tile).
-bool skips_empty(rick_handle h) { return h->strip && h->chunks.size() <= (size_t)kMaxChunksPerPass; }
+bool skips_empty(rick_handle h) { return (h->strip || h->longrows) && h->chunks.size() <= (size_t)kMaxChunksPerPass; }
 
 ChunkList chunk_list(rick_handle h, size_t c0)
 {
@@ -406,21 +413,23 @@ void strip_free(rick_handle h)
     h->sargs = StripArgs{};
 }
 
-// Buffers and twiddles of the strip transform (rick_create); false where they
-// do not fit.
-bool strip_alloc(rick_handle h)
+// Buffers and twiddles of the strip transform, or of the split transform's
+// sparse rows (rick_create); false where they do not fit.
+bool strip_alloc(rick_handle h, bool strip)
 {
     const GridCfg& c = h->cfg;
     const size_t pb = plane_bytes(&h->p);
     const int n = h->p.n, r = n / 256, wpr = (c.ntu + 31) / 32;
     size_t fr = 0, tot = 0;
     const size_t bits = (size_t)c.nw * c.ntu * wpr * sizeof(uint32_t), rng = (size_t)c.nw * sizeof(int2);
-    const size_t t1 = 15 * (size_t)(n / 16), t2 = 15 * (size_t)r, tw = (t1 + t2) * sizeof(float2);
-    const size_t tab = (size_t)h->nchan * (n / 2 + 1) * (n / 2 + 16);  // entries of each screen table
-    const size_t tab_bytes = 3 * tab * sizeof(float2);
-    const size_t need = (size_t)h->G * pb + bits + rng + tw + tab_bytes;
+    const int q = strip ? 0 : n / 4096;
+    const size_t t1 = 15 * (size_t)(n / 16), t2 = 15 * (size_t)r, tw = (t1 + t2 + 15 * (size_t)q) * sizeof(float2);
+    // entries of each screen table
+    const size_t tab = strip ? (size_t)h->nchan * (n / 2 + 1) * (n / 2 + 16) : 0;
+    const size_t tab_bytes = 3 * tab * sizeof(float2), strip_bytes = strip ? (size_t)h->G * pb : 0;
+    const size_t need = strip_bytes + bits + rng + tw + tab_bytes;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || need + (64u << 20) > fr) return false;
-    std::vector<float2> w(t1 + t2);
+    std::vector<float2> w(tw / sizeof(float2));
     for (int k = 1; k < 16; ++k) {
         for (int j = 0; j < n / 16; ++j) {
             const double a = 6.283185307179586476925 * (double)((int64_t)j * k % n) / (double)n;
@@ -430,24 +439,30 @@ bool strip_alloc(rick_handle h)
             const double a = 6.283185307179586476925 * (double)(j * k % (n / 16)) / (double)(n / 16);
             w[t1 + (k - 1) * r + j] = make_float2((float)std::cos(a), (float)std::sin(a));
         }
+        for (int j = 0; j < q; ++j) {
+            const double a = 6.283185307179586476925 * (double)(j * k) / (double)r;
+            w[t1 + t2 + (k - 1) * q + j] = make_float2((float)std::cos(a), (float)std::sin(a));
+        }
     }
     float2* dev_tw = nullptr;
-    bool ok = cudaMalloc((void**)&h->strips, (size_t)h->G * pb) == cudaSuccess &&
+    bool ok = (!strip || cudaMalloc((void**)&h->strips, strip_bytes) == cudaSuccess) &&
               cudaMalloc((void**)&h->sargs.bits, bits) == cudaSuccess &&
               cudaMalloc((void**)&h->sargs.range, rng) == cudaSuccess &&
-              cudaMalloc((void**)&h->sargs.tab.rho, tab_bytes) == cudaSuccess &&
+              (!strip || cudaMalloc((void**)&h->sargs.tab.rho, tab_bytes) == cudaSuccess) &&
               cudaMalloc((void**)&dev_tw, tw) == cudaSuccess;
     h->sargs.tw1 = dev_tw;
     h->sargs.tw2 = dev_tw ? dev_tw + t1 : nullptr;
-    h->sargs.tab.kap = h->sargs.tab.rho + tab;
-    h->sargs.tab.fin = h->sargs.tab.kap + tab;
     ok = ok && cudaMemcpy(dev_tw, w.data(), tw, cudaMemcpyHostToDevice) == cudaSuccess;
-    ok = ok && encode_rows_map(h->rowsmap, h->strips, n, h->G) == cudaSuccess;
-    h->sargs.map = h->rowsmap;
-    StackArgs a = stack_args(h);
-    if (h->batch) a.chan_screen = h->chan_scr;
-    h->screen_k0 = 0;
-    ok = ok && launch_screen(h->sargs, a, h->taper, true, h->nchan, nullptr) == cudaSuccess;
+    if (ok && strip) {
+        h->sargs.tab.kap = h->sargs.tab.rho + tab;
+        h->sargs.tab.fin = h->sargs.tab.kap + tab;
+        ok = encode_rows_map(h->rowsmap, h->strips, n, h->G) == cudaSuccess;
+        h->sargs.map = h->rowsmap;
+        StackArgs a = stack_args(h);
+        if (h->batch) a.chan_screen = h->chan_scr;
+        h->screen_k0 = 0;
+        ok = ok && launch_screen(h->sargs, a, h->taper, true, h->nchan, nullptr) == cudaSuccess;
+    }
     if (!ok) {
         (void)cudaGetLastError();
         strip_free(h);
@@ -793,7 +808,8 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
             for (int j = 0; j < kPolyTerms; ++j) h->cfg.coef[t][j] = (t < c.S) ? coef[t * kPolyTerms + j] : 0.0f;
         set_tap_sum(h->cfg);
     }
-    h->strip = want_strip(*p) && h->amp <= kStripAmp && strip_alloc(h);
+    h->strip = want_strip(*p) && h->amp <= kStripAmp && strip_alloc(h, true);
+    h->longrows = want_longrows(*p) && h->amp <= kLongAmp && strip_alloc(h, false);
     // the cuFFT plans this handle's transform path uses
     if (!h->strip) {
         cufftHandle plan;
@@ -808,11 +824,13 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
         h->cfg.row_perm = 0;
         if (split)
             while ((1 << h->cfg.row_perm) < n1) ++h->cfg.row_perm;
-        s = get_plan(h, G, &plan, kind);
-        if (s) return cleanup(s);
-        if (NW % G) {
-            s = get_plan(h, NW % G, &plan, kind);
+        if (!h->longrows) {  // whose rows are the library's own
+            s = get_plan(h, G, &plan, kind);
             if (s) return cleanup(s);
+            if (NW % G) {
+                s = get_plan(h, NW % G, &plan, kind);
+                if (s) return cleanup(s);
+            }
         }
     }
     if (h->batch_split) {
@@ -1003,7 +1021,7 @@ rick_status rick_fft_and_stack(rick_handle h, float* image)
     const bool split = use_split(p, &n1, &n2);
     const int lo = h->cfg.plane_lo, hi = h->cfg.plane_hi;
     StripArgs sa = h->sargs;
-    if (h->strip) {  // the tiles and rows the transform works on
+    if (h->strip || h->longrows) {  // the tiles and rows the transform works on
         ChunkList cl = chunk_list(h, 0);
         if (!skips_empty(h)) cl.count = -1;
         PhaseScope fs(h, kPhasePrep);
@@ -1030,17 +1048,22 @@ rick_status rick_fft_and_stack(rick_handle h, float* image)
             if ((s = strip_screen(h, a, k0))) return s;
             RICK_CU(h, launch_colimage(sa, a, h->strips, h->acc, norm_sum(h), image, &h->ctr->err, h->stream));
         } else if (split) {
-            cufftHandle rows;
-            if ((s = get_plan(h, nk, &rows, kPlanRows))) return s;
             if ((s = colfft_ready(h))) return s;
-            {
+            if (h->longrows) {
+                PhaseScope fs(h, kPhaseFft);
+                RICK_CU(h, launch_longrows(p.n, +1, sa, k0, nk, h->cfg.row_perm, h->planes, h->stream));
+                count_launches(h, 1);
+            } else {
+                cufftHandle rows;
+                if ((s = get_plan(h, nk, &rows, kPlanRows))) return s;
                 PhaseScope fs(h, kPhaseFft);
                 RICK_FFT(h, cufftExecC2C(rows, planes, planes, CUFFT_INVERSE));
             }
             {
                 PhaseScope cs(h, kPhaseColfft);
-                RICK_CU(h, launch_colfft(h->cfmap, h->cf_tw, h->planes, p.n, nk, +1, h->dbg_wait_ns, &h->ctr->err,
-                                         h->stream));
+                RICK_CU(h, launch_colfft(h->cfmap, h->cf_tw, h->planes, p.n, nk, +1,
+                                         h->longrows ? sa.range + k0 : nullptr, h->cfg.log2T, h->dbg_wait_ns,
+                                         &h->ctr->err, h->stream));
                 count_launches(h, 1);
             }
             if (!h->colmap_ready) {
@@ -1113,7 +1136,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
     const bool split = use_split(p, &n1, &n2);
     cufftComplex* planes = reinterpret_cast<cufftComplex*>(h->planes);
     StripArgs sa = h->sargs;
-    if (!st && h->strip) {  // the tiles that the footprints touch
+    if (!st && (h->strip || h->longrows)) {  // the tiles that the footprints touch
         ChunkList cl{};
         cl.off[0] = off;
         cl.count = 1;
@@ -1148,16 +1171,21 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
         }
         cufftResult r = CUFFT_SUCCESS;
         if (split) {
-            cufftHandle rows;
-            if ((st = get_plan(h, nk, &rows, kPlanRows))) break;
             if ((st = colfft_ready(h))) break;
-            e = launch_colfft(h->cfmap, h->cf_tw, h->planes, p.n, nk, -1, h->dbg_wait_ns, &h->ctr->err, h->stream);
+            e = launch_colfft(h->cfmap, h->cf_tw, h->planes, p.n, nk, -1, h->longrows ? sa.range + k0 : nullptr,
+                              c.log2T, h->dbg_wait_ns, &h->ctr->err, h->stream);
+            if (e == cudaSuccess && h->longrows)
+                e = launch_longrows(p.n, -1, sa, k0, nk, c.row_perm, h->planes, h->stream);
             if (e != cudaSuccess) {
                 st = fail(h, RICK_ERR_CUDA, "k_colfft: %s", cudaGetErrorString(e));
                 break;
             }
-            count_launches(h, 1);
-            r = cufftExecC2C(rows, planes, planes, CUFFT_FORWARD);
+            count_launches(h, h->longrows ? 2 : 1);
+            if (!h->longrows) {
+                cufftHandle rows;
+                if ((st = get_plan(h, nk, &rows, kPlanRows))) break;
+                r = cufftExecC2C(rows, planes, planes, CUFFT_FORWARD);
+            }
         } else {
             cufftHandle plan;
             if ((st = get_plan(h, nk, &plan))) break;
@@ -1428,7 +1456,7 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
         RICK_CU(h, launch_scatter(c, u, v, w, weights, vis2, m, nullptr, h->cursor, h->b_ent, h->ctr, h->chan_sw,
                                   h->stream));
         count_launches(h, 5);
-        if (h->strip) {
+        if (h->strip || h->longrows) {
             ChunkList cl{};
             cl.off[0] = h->b_off;
             cl.count = 1;
@@ -1476,12 +1504,16 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
             count_launches(h, 2);
             return RICK_OK;
         }
-        cufftHandle rows;
-        rick_status s = get_plan(h, nk, &rows, kPlanRows);
-        if (s) return s;
         int n1 = 0, n2 = 0;
         colstack_shape(p.n, &n1, &n2);
-        {
+        if (h->longrows) {
+            PhaseScope fs(h, kPhaseFft);
+            RICK_CU(h, launch_longrows(p.n, +1, h->sargs, k0, nk, c.row_perm, buf, st));
+            count_launches(h, 1);
+        } else {
+            cufftHandle rows;
+            rick_status s = get_plan(h, nk, &rows, kPlanRows);
+            if (s) return s;
             PhaseScope fs(h, kPhaseFft);
             RICK_FFT(h, cufftSetStream(rows, st));
             RICK_FFT(h, cufftExecC2C(rows, reinterpret_cast<cufftComplex*>(buf), reinterpret_cast<cufftComplex*>(buf),
@@ -1489,8 +1521,9 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
         }
         {
             PhaseScope cs(h, kPhaseColfft);
-            RICK_CU(h, launch_colfft(b ? h->cfmap2 : h->cfmap, h->cf_tw, buf, p.n, nk, +1, h->dbg_wait_ns,
-                                     &h->ctr->err, st));
+            RICK_CU(h, launch_colfft(b ? h->cfmap2 : h->cfmap, h->cf_tw, buf, p.n, nk, +1,
+                                     h->longrows ? h->sargs.range + k0 : nullptr, c.log2T, h->dbg_wait_ns, &h->ctr->err,
+                                     st));
             count_launches(h, 1);
         }
         // one launch over the group's channels (grid z = channel)
@@ -1517,7 +1550,7 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
         cl.off[0] = h->b_off;
         cl.ent[0] = h->b_ent;
         cl.count = 1;
-        RICK_CU(h, launch_grid(c, cl, k0, nk, true, false, h->b_heavy, h->b_heavy_words, buf, h->stream, h->strip));
+        RICK_CU(h, launch_grid(c, cl, k0, nk, true, false, h->b_heavy, h->b_heavy_words, buf, h->stream, h->strip || h->longrows));
         count_launches(h, 2);
         return RICK_OK;
     };
@@ -1643,7 +1676,8 @@ rick_status rick_image_batch(rick_handle h, const float* vis, const float* u, co
         // per plane group the two gridder kernels, then k_colfft and one
         // k_colstack over its channels (split) or one k_stack over them
         const int groups = (c.nw + h->G - 1) / h->G;
-        count_launches(h, h->strip ? 6 + 4 * groups : 5 + (h->batch_split ? 4 : 3) * groups);
+        count_launches(h, h->strip ? 6 + 4 * groups
+                                   : h->longrows ? 6 + 5 * groups : 5 + (h->batch_split ? 4 : 3) * groups);
         return RICK_OK;
     }
     if (!use_graph) return batch_body(h, vis, u, v, w, weights, m, images);

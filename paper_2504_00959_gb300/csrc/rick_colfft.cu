@@ -45,7 +45,7 @@ namespace {
 
 constexpr int kCfThreads = 256;
 constexpr unsigned long long kCfWaitNs = 1000000000ull;  // bound of the load wait: 1 s
-constexpr int kCfBoxRows = 256;                          // TMA box: at most 256 rows per copy
+constexpr int kCfBoxRows = 128;  // TMA box: rows per copy (the unit in which empty rows are left out)
 
 __device__ __forceinline__ float2 c_add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 c_sub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
@@ -174,7 +174,7 @@ __device__ __forceinline__ float2 twid(const float2* tw, int e)
 // ([N1][W] complex values), output f1 written to row f1 of the run at P.
 template <int N1, int W, int SIGN>
 __device__ __forceinline__ void colfft_two_pass(float2* __restrict__ buf, const float2* tw,
-                                                float2* __restrict__ P, int n, int t)
+                                                float2* __restrict__ P, int n, int t, int alo, int ahi)
 {
     constexpr int Q = N1 / 16;
     // pass A: 16-point DFTs over a1 (rows Q a1 + a2), twiddle w_N1^(a2 k1)
@@ -182,7 +182,11 @@ __device__ __forceinline__ void colfft_two_pass(float2* __restrict__ buf, const 
         const int x = it % W, a2 = it / W;
         float2 v[16];
 #pragma unroll
-        for (int a1 = 0; a1 < 16; ++a1) v[a1] = buf[(Q * a1 + a2) * W + x];
+        for (int a1 = 0; a1 < 16; ++a1) {
+            const int a = Q * a1 + a2;
+            // imaging: rows outside the plane's range are zero (and were not copied)
+            v[a1] = SIGN < 0 || (a >= alo && a < ahi) ? buf[a * W + x] : make_float2(0.f, 0.f);
+        }
         dft16<SIGN>(v);
 #pragma unroll
         for (int k1 = 0; k1 < 16; ++k1) {
@@ -197,14 +201,17 @@ __device__ __forceinline__ void colfft_two_pass(float2* __restrict__ buf, const 
         for (int it = t; it < 16 * W; it += kCfThreads) {
             const int x = it % W, k1 = it / W;
             if constexpr (Q == 1) {
-                P[(size_t)k1 * n + x] = buf[k1 * W + x];
+                P[(size_t)k1 * n + x] = buf[k1 * W + x];  // n = 256: always the whole range
             } else {
                 float2 v[Q];
 #pragma unroll
                 for (int a2 = 0; a2 < Q; ++a2) v[a2] = buf[(Q * k1 + a2) * W + x];
                 dft_small<Q, SIGN>(v);
 #pragma unroll
-                for (int kq = 0; kq < Q; ++kq) P[(size_t)(k1 + 16 * kq) * n + x] = v[kq];
+                for (int kq = 0; kq < Q; ++kq) {
+                    const int f1 = k1 + 16 * kq;
+                    if (SIGN > 0 || (f1 >= alo && f1 < ahi)) P[(size_t)f1 * n + x] = v[kq];
+                }
             }
         }
     } else {
@@ -245,8 +252,10 @@ __device__ __forceinline__ void colfft_two_pass(float2* __restrict__ buf, const 
             for (int q = 0; q < r; ++q) v[q] = buf[(Q * k1 + 16 * q + (j1 ^ q)) * W + xx];
             dft_small<r, SIGN>(v);
 #pragma unroll
-            for (int j2 = 0; j2 < r; ++j2)
-                P[(size_t)(k1 + 16 * (j1 + 16 * j2)) * n + xx] = v[j2];
+            for (int j2 = 0; j2 < r; ++j2) {
+                const int f1 = k1 + 16 * (j1 + 16 * j2);
+                if (SIGN > 0 || (f1 >= alo && f1 < ahi)) P[(size_t)f1 * n + xx] = v[j2];
+            }
         }
     }
 }
@@ -255,10 +264,15 @@ __device__ __forceinline__ void colfft_two_pass(float2* __restrict__ buf, const 
 // memory N1 * W complex values, the N1 twiddles and one mbarrier.  tw:
 // exp(+2 pi i j / N1), j < N1 (device; copied in with the block's data).
 // err: bit 1 set when the load wait ran out.
+// range (or NULL: all): the tile rows [lo, hi) of each plane that hold anything
+// (imaging: the other rows are taken as zeros and not read) or are wanted
+// (adjoint: the other rows are not written); tile sides are multiples of 16,
+// so the rows 16 a + b of every b have the same range of a.
 template <int N1, int W, int SIGN>
 __global__ void __launch_bounds__(kCfThreads) k_colfft(const __grid_constant__ CUtensorMap map,
                                                        const float2* __restrict__ tw, float2* __restrict__ planes,
-                                                       int n, unsigned long long wait_ns,
+                                                       int n, const int2* __restrict__ range, int log2T,
+                                                       unsigned long long wait_ns,
                                                        unsigned long long* __restrict__ err)
 {
     constexpr int kBox = N1 < kCfBoxRows ? N1 : kCfBoxRows;
@@ -271,6 +285,13 @@ __global__ void __launch_bounds__(kCfThreads) k_colfft(const __grid_constant__ C
     const int t = threadIdx.x;
     const int x0 = blockIdx.x * W, b = blockIdx.y, plane = blockIdx.z;
     const unsigned long long limit = wait_ns ? wait_ns : kCfWaitNs;
+    int alo = 0, ahi = N1;
+    if (range) {
+        const int2 rg = __ldg(range + plane);
+        alo = (rg.x << log2T) >> 4;
+        ahi = (rg.y << log2T) >> 4;
+        if (SIGN < 0 && ahi <= alo) return;  // nothing wanted of this plane
+    }
     if (t == 0) {
         s_abort = 0;
         mbar_init(smem_u32(bar), 1);
@@ -278,9 +299,11 @@ __global__ void __launch_bounds__(kCfThreads) k_colfft(const __grid_constant__ C
     }
     __syncthreads();
     if (t == 0) {
-        mbar_expect(smem_u32(bar), (uint32_t)((N1 * W + N1) * sizeof(float2)));
-#pragma unroll
-        for (int a0 = 0; a0 < N1; a0 += kBox)
+        // imaging: the boxes of rows that meet the range
+        const int first = SIGN > 0 ? alo / kBox * kBox : 0, last = SIGN > 0 ? ahi : N1;
+        const int boxes = last > first ? (last - first + kBox - 1) / kBox : 0;
+        mbar_expect(smem_u32(bar), (uint32_t)((boxes * kBox * W + N1) * sizeof(float2)));
+        for (int a0 = first; a0 < last; a0 += kBox)
             tma_load_3d(smem_u32(buf + (size_t)a0 * W), &map, x0, a0, plane * 16 + b, smem_u32(bar));
         bulk_load(smem_u32(tws), tw, (uint32_t)(N1 * sizeof(float2)), smem_u32(bar));
     }
@@ -312,13 +335,13 @@ __global__ void __launch_bounds__(kCfThreads) k_colfft(const __grid_constant__ C
             for (int f1 = 0; f1 < N1; ++f1) P[(size_t)f1 * n + it] = v[f1];
         }
     } else {
-        colfft_two_pass<N1, W, SIGN>(buf, tws, P, n, t);
+        colfft_two_pass<N1, W, SIGN>(buf, tws, P, n, t, alo, ahi);
     }
 }
 
 template <int N1, int W, int SIGN>
-cudaError_t launch_cf(const void* map, const float2* tw, float2* planes, int n, int nk, unsigned long long wait_ns,
-                      unsigned long long* err, cudaStream_t s)
+cudaError_t launch_cf(const void* map, const float2* tw, float2* planes, int n, int nk, const int2* range, int log2T,
+                      unsigned long long wait_ns, unsigned long long* err, cudaStream_t s)
 {
     const size_t smem = (size_t)(N1 * W + N1) * sizeof(float2) + 16;
     static bool attr_done[64] = {false};
@@ -332,7 +355,7 @@ cudaError_t launch_cf(const void* map, const float2* tw, float2* planes, int n, 
     }
     const dim3 grid((unsigned)(n / W), 16u, (unsigned)nk);
     k_colfft<N1, W, SIGN><<<grid, kCfThreads, smem, s>>>(*reinterpret_cast<const CUtensorMap*>(map), tw, planes,
-                                                          n, wait_ns, err);
+                                                          n, range, log2T, wait_ns, err);
     return cudaGetLastError();
 }
 
@@ -378,16 +401,16 @@ cudaError_t encode_colfft_map(void* map, const float2* planes, int n, int planes
 }
 
 cudaError_t launch_colfft(const void* map, const float2* tw, float2* planes, int n, int nk, int sign,
-                          unsigned long long wait_ns, unsigned long long* err, cudaStream_t s)
+                          const int2* range, int log2T, unsigned long long wait_ns, unsigned long long* err, cudaStream_t s)
 {
     if (nk <= 0) return cudaSuccess;
     if (nk > 65535) return cudaErrorInvalidValue;
     const int n1 = n / 16;
 #define RICK_CF_CASE(N1)                                                                                   \
     case N1:                                                                                               \
-        return sign > 0 ? launch_cf<N1, cf_width<N1>(), 1>(map, tw, planes, n, nk, wait_ns, err, s)        \
-                        : launch_cf<N1, cf_width<N1>(), -1>(map, tw, planes, n, nk, wait_ns, err, s);
-    if (n != 16 * n1) return cudaErrorInvalidValue;
+        return sign > 0 ? launch_cf<N1, cf_width<N1>(), 1>(map, tw, planes, n, nk, range, log2T, wait_ns, err, s)        \
+                        : launch_cf<N1, cf_width<N1>(), -1>(map, tw, planes, n, nk, range, log2T, wait_ns, err, s);
+    if (n != 16 * n1 || (range && n1 < 16)) return cudaErrorInvalidValue;
     switch (n1) {
         RICK_CF_CASE(4)
         RICK_CF_CASE(8)

@@ -330,8 +330,9 @@ cudaError_t launch_colstack(const void* map, const StackArgs& a, int n1, int n2,
 // N1 = n / 16-point DFT with exponent sign (+1 imaging, -1 adjoint); map
 // from encode_colfft_map for the plane buffer, tw = exp(+2 pi i j / N1)
 cudaError_t encode_colfft_map(void* map, const float2* planes, int n, int planes_in_buffer);
+// range (of the group's planes; NULL: all rows): see k_colfft
 cudaError_t launch_colfft(const void* map, const float2* tw, float2* planes, int n, int nk, int sign,
-                          unsigned long long wait_ns, unsigned long long* err, cudaStream_t s);
+                          const int2* range, int log2T, unsigned long long wait_ns, unsigned long long* err, cudaStream_t s);
 cudaError_t launch_spreadcol(const StackArgs& a, int n1, int n2, const void* rimg, const float* taper,
                              const double* sum_w, float2* planes, cudaStream_t s);
 
@@ -376,6 +377,13 @@ cudaError_t launch_colspread(const StripArgs& s, const StackArgs& a, const void*
                              float2* strips, cudaStream_t st);
 
 // nchan > 1: channels a.chan0 .. of a batch in one launch (as launch_colstack)
+// ---- sparse rows of the split transform, n = 8192 and 16384 (rick_longrow.cu):
+// in place, bits / range / twiddles as above with tw1 w_n^(j k1) [15][n / 16],
+// tw2 w_(n/16)^(t2 k2) [15][n / 256], then w_(n/256)^(s k3) [15][n / 4096]
+bool longrow_shape(int n);
+cudaError_t launch_longrows(int n, int dir, const StripArgs& s, int k0, int nk, int row_perm, float2* planes,
+                            cudaStream_t st);
+
 cudaError_t launch_stack(const StackArgs& a, const float2* planes, float2* acc, const float* taper,
                          const double* sum_w, void* image, cudaStream_t s, int nchan = 1);
 
@@ -453,6 +461,7 @@ struct rick_imager {
     // the two-pass transform (rick_strip.cu): the strip buffer of a group, the
     // tile bits and row ranges of every plane, and the twiddles
     double amp;                      // what the grid correction does to rounding: mean 1 / taper^2 (1 without)
+    bool longrows;                   // the split transform with sparse rows (rick_longrow.cu)
     bool strip;
     float2* strips;                  // [G][n / 2][n] pairs of columns
     rick::StripArgs sargs;

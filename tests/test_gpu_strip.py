@@ -1,6 +1,6 @@
 """The two-pass transform of n = 1024, 2048, 4096 (row transforms of the
 non-empty tiles, then the whole column transform with the w-screen and the
-plane sum) against cuFFT's 2D plan and the separate stack (RICK_FFT_2D), where
+plane sum) and the split transform's sparse rows of n = 8192, 16384 against cuFFT's 2D plan and the separate stack (RICK_FFT_2D), where
 its work depends on the data: empty tiles, tile rows and planes, every tile
 side, several plane groups and more planes than one run of the screen's
 rotation, several chunks of measurements (their tiles united; more than one
@@ -77,6 +77,9 @@ def _same(a, b, tol):
     (4096, 4, 300, 32, {"part": 0.9, "S": 8}),         # mostly empty tiles
     (4096, 2, 50000, 16, {"part": 0.1}),
     (4096, 33, 40000, 64, {"empty_planes": True}),     # one plane past a run
+    (8192, 4, 20000, 16, {"empty_planes": True}),      # the split transform's sparse rows
+    (8192, 2, 2000, 64, {"part": 0.3}),
+    (16384, 2, 20000, 32, {"part": 0.5, "empty_planes": True}),
 ])
 def test_equals_2d_plan(rick, n, nw, m, tile, extra):
     p, data = _problem(n, nw, m, 11 + n + nw + tile, **extra)
