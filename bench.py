@@ -376,7 +376,7 @@ def main():
                     help="planes per measurement (Eq. 3's kernel in w); the plane range is padded by "
                          "nw / (nw - w_support) so every footprint lies on the planes")
     ap.add_argument("--fft2d", action="store_true",
-                    help="cuFFT's 2D plan + a separate stack pass (RICK_FFT_2D) instead of the split transform")
+                    help="cuFFT's 2D plan + a separate stack pass (RICK_FFT_2D) instead of the library's transforms")
     ap.add_argument("--no-cpu-baseline", action="store_true",
                     help="skip the FP64 oracle (CPU baseline and parity of the timed image)")
     ap.add_argument("--no-e2e", action="store_true", help="skip the host-buffer end-to-end leg")
@@ -427,6 +427,37 @@ def _nvml_for(dev):
     uuid = str(getattr(props, "uuid", ""))
     uuid = uuid if uuid.startswith("GPU-") else ("GPU-" + uuid if uuid else "")
     return (Nvml(uuid) if uuid else None), (uuid if uuid else dev.index)
+
+
+def occupancy(prob, params, tile, k0, k1):
+    """Share of the tiles of planes k0 .. k1-1 that hold any footprint, and of
+    the rows in each plane's range of non-empty tile rows: what the gridder and
+    the library's own row transforms move.  (1, 1) with w-support, whose
+    footprints are not followed here."""
+    import torch
+    if params.get("w_support", 1) > 1:
+        return 1.0, 1.0
+    n, nw, S = params["n"], params["nw"], params["support"]
+    nt = -(-n // tile)
+    full = torch.zeros(nw * nt * nt, dtype=torch.bool, device=prob["u"].device)
+    scale, dw = n * params["pixel_rad"], (params["w_max"] - params["w_min"]) / nw
+    for a in range(0, prob["u"].numel(), 1 << 24):
+        u, v, w = (prob[x][a:a + (1 << 24)] for x in "uvw")
+        if params["flags"] & 32:  # Hermitian fold
+            s = torch.where(w < 0, -1.0, 1.0)
+            u, v, w = u * s, v * s, w * s
+        fu, fv = (torch.floor(x * scale + n // 2 - 0.5 * S).long() + 1 for x in (u, v))
+        k = torch.floor((w - params["w_min"]) / dw).long().clamp(0, nw - 1)
+        ok = (fu >= 0) & (fu + S <= n) & (fv >= 0) & (fv + S <= n)
+        fu, fv, k = fu[ok], fv[ok], k[ok]
+        for du in (0, S - 1):
+            for dv in (0, S - 1):
+                full[(k * nt + (fv + dv) // tile) * nt + (fu + du) // tile] = True
+    rows = full.view(nw, nt, nt)[k0:k1].any(2)
+    idx = torch.arange(nt, device=rows.device)
+    lo = torch.where(rows, idx, nt).amin(1)
+    hi = torch.where(rows, idx + 1, 0).amax(1)
+    return float(full.view(nw, -1)[k0:k1].float().mean()), float((hi - lo).clamp(min=0).float().mean() / nt)
 
 
 def run_image(args, rank, world):
@@ -513,31 +544,38 @@ def run_image(args, rank, world):
 
     # ------------------------------------------------ rooflines and phases
     # algorithmic bytes per step: the gridder reads each gridded measurement
-    # once (u, v, w, weight, visibility: 24 B) and writes every plane cell
-    # once (8 B); cuFFT at least two read + write passes over the planes;
-    # the stack reads every plane once and writes the image (4 B per pixel,
-    # plus the complex accumulator between plane groups); the prep reads the
-    # measurements twice (count, scatter; a third time for the uniform-
-    # weighting density) and writes one 16 B entry per (measurement, tile)
+    # once (u, v, w, weight, visibility: 24 B) and writes every cell of the
+    # non-empty tiles once (8 B; with cuFFT's 2D plan every cell); the row
+    # transforms read those and write the rows of each plane's non-empty range;
+    # the column factor reads those and writes every cell, and the column
+    # transform fused with the stack reads them (the fused last factor: every
+    # cell) and writes the image (4 B per pixel, plus the complex accumulator
+    # between plane groups); cuFFT's 2D plan at least two read + write passes;
+    # the prep reads the measurements twice (count, scatter; a third time for
+    # the uniform-weighting density) and writes one 16 B entry per
+    # (measurement, tile)
     peak, peak_kind = _peaks()
     cells = float(k1 - k0) * n * n  # this rank's planes
     groups = -(-(k1 - k0) // max(st["plane_group"], 1))
     uniform = bool(params["flags"] & synth.FLAG_UNIFORM)
     grid_ms = tm["grid_ms"] / steps
-    grid_bytes = 24.0 * st["n_gridded"] + 8.0 * cells
+    split = tm["colfft_calls"] > 0  # the split transform: k_longrows (n >= 8192), k_colfft, k_colstack
+    strip = not split and not args.fft2d and n in (1024, 2048, 4096)  # k_rows, k_colimage
+    tiles, rows = (1.0, 1.0) if args.fft2d else occupancy(prob, params, st["tile"], k0, k1)
+    grid_bytes = 24.0 * st["n_gridded"] + 8.0 * cells * tiles
     stack_ms = tm["stack_ms"] / steps
-    stack_bytes = 8.0 * cells + 4.0 * n * n + (2 * 8.0 * n * n * (groups - 1) if groups > 1 else 0.0)
-    split = tm["colfft_calls"] > 0  # the split transform: cuFFT rows, k_colfft, k_colstack
+    stack_bytes = (8.0 * cells * (rows if strip else 1.0) + 4.0 * n * n +
+                   (2 * 8.0 * n * n * (groups - 1) if groups > 1 else 0.0))
     fft_ms = tm["fft_ms"] / steps
-    fft_bytes = (1 if split else 2) * 2 * 8.0 * cells  # one read + write pass per dimension
+    fft_bytes = 8.0 * cells * (tiles + rows) if split or strip else 4 * 8.0 * cells
     colfft_ms = tm["colfft_ms"] / steps
-    colfft_bytes = 2 * 8.0 * cells if split else 0.0
+    colfft_bytes = 8.0 * cells * (rows + 1.0) if split else 0.0
     prep_ms = tm["prep_ms"] / steps
     prep_bytes = (3 if uniform else 2) * 24.0 * m + 16.0 * st["n_entries"]
     phases = {
         "prep": {"ms": prep_ms, "algorithmic_gb": prep_bytes / 1e9},
         "grid": {"ms": grid_ms, "algorithmic_gb": grid_bytes / 1e9},
-        ("fft_cufft_rows" if split else "fft_cufft"): {"ms": fft_ms, "algorithmic_gb": fft_bytes / 1e9},
+        ("fft_rows" if split or strip else "fft_cufft"): {"ms": fft_ms, "algorithmic_gb": fft_bytes / 1e9},
         "stack": {"ms": stack_ms, "algorithmic_gb": stack_bytes / 1e9},
     }
     if split:
@@ -552,9 +590,10 @@ def run_image(args, rank, world):
     default_size = wl == "wstack" and (n, nw, m) == (4096, 32, 10_000_000) and plain
     large_size = wl == "large" and (n, nw, m) == (16384, 128, 200_000_000) and plain
     traffic = _traffic("rick_grid.cu", "k_grid@4096x32x1e7") if default_size else None
-    stack_name = ("k_colstack (last 16-point column factor + w-screen + stack, Eq. 1)" if split
+    stack_name = ("k_colimage (column transform + w-screen + stack, Eq. 1)" if strip else
+                  "k_colstack (last 16-point column factor + w-screen + stack, Eq. 1)" if split
                   else "k_stack (w-screen + stack, Eq. 1)")
-    stack_traffic = _traffic("rick_stack.cu", "k_colstack@4096x32x1e7") if (default_size and split) else None
+    stack_traffic = _traffic("rick_strip.cu", "k_colimage@4096x32x1e7") if (default_size and strip) else None
     launches_grid = max(tm["grid_calls"] / steps, 1)
     launches_stack = max(tm["stack_calls"] / steps, 1)
     rl_grid = {"kernel": "k_grid_tiles + k_grid_heavy (gridding, Eq. 3)", "bound": "hbm",
@@ -567,6 +606,14 @@ def run_image(args, rank, world):
                 "peak_kind": peak_kind, "algorithmic_bytes_per_launch": stack_bytes / launches_stack,
                 "launch_ms": stack_ms / launches_stack, "launches_per_step": launches_stack}
     own = [(grid_ms, rl_grid), (stack_ms, rl_stack)]
+    if split or strip:
+        launches_rows = max(tm["fft_calls"] / steps, 1)
+        own.append((fft_ms, {
+            "kernel": "k_rows / k_longrows (row transforms of the non-empty tiles and rows)", "bound": "hbm",
+            "achieved": fft_bytes / fft_ms / 1e6, "peak": peak, "unit": "GB/s", "frac": fft_bytes / fft_ms / 1e6 / peak,
+            "traffic": _traffic("rick_strip.cu", "k_rows@4096x32x1e7") if (default_size and strip) else None,
+            "peak_kind": peak_kind, "algorithmic_bytes_per_launch": fft_bytes / launches_rows,
+            "launch_ms": fft_ms / launches_rows, "launches_per_step": launches_rows}))
     if split:
         launches_cf = max(tm["colfft_calls"] / steps, 1)
         own.append((colfft_ms, {
@@ -668,7 +715,7 @@ def run_image(args, rank, world):
         energy = (e1 - e0) / 1e3 / steps
 
     config = workload_config(wl, params, m, world, args)
-    # whole step against HBM: prep + gridder + FFT (2 passes) + stack
+    # whole step against HBM: prep + gridder + transform + stack
     step_bytes = prep_bytes + grid_bytes + fft_bytes + colfft_bytes + stack_bytes
     out = {
         "metric": METRIC, "value": value, "unit": "vis/s", "n_gpus": world, "steps": args.steps,
@@ -679,7 +726,8 @@ def run_image(args, rank, world):
         "energy_j_per_solution": energy, "e2e": e2e, "cpu_baseline": cpu, "parity": parity,
         "gpu_launches": int(tm["kernel_launches"]), "clocks": clk,
         "launch": {"tile": st["tile"], "plane_group": st["plane_group"], "plane_groups": groups,
-                   "planes_of_rank0": [k0, k1], "workspace_gb": st["workspace_bytes"] / 1e9},
+                   "planes_of_rank0": [k0, k1], "tiles_non_empty": tiles, "rows_in_range": rows,
+                   "workspace_gb": st["workspace_bytes"] / 1e9},
     }
     if rank == 0:
         print(json.dumps(out))
@@ -782,7 +830,8 @@ def run_channels(args, rank, world):
         return f0.elapsed_time(f1) / ksteps, k0, k1
 
     # the per-channel loop with the library's default single-image path, and
-    # with the split transform (the batch's); the faster one is the reference
+    # with RICK_FFT_SPLIT (which only sizes outside 1024 .. 4096 tell apart);
+    # the faster one is the reference
     t_loop, k0, k1 = time_loop()
     loop_default = loop_out.clone()
     for im in ims:
@@ -881,11 +930,14 @@ def run_adjoint(args, rank, world):
     tm = im.timing()
     st = im.stats()
     peak, peak_kind = _peaks()
-    # backward = spread (8 B/cell written) + forward FFT (two passes, read +
-    # write) + gather (planes read once, 16 B of u, v, w, weight + 8 B of
-    # gradient per measurement) + the measurement sort (two passes of 16 B)
+    # backward = column transforms of the image's spread (they write every
+    # cell of the rows that a gather reads) + row transforms (those rows read,
+    # the non-empty tiles written) + gather (the non-empty tiles read, 16 B of
+    # u, v, w, weight + 8 B of gradient per measurement) + the measurement
+    # sort (two passes of 16 B)
     deg_ms = tm["degrid_ms"] / max(tm["degrid_calls"], 1)
-    deg_bytes = 8.0 * nw * n * n + 32.0 * nw * n * n + 8.0 * nw * n * n + 24.0 * m + 32.0 * m
+    tiles, rows = occupancy(prob, params, st["tile"], 0, nw)
+    deg_bytes = 8.0 * nw * n * n * (2 * rows + 2 * tiles) + 24.0 * m + 32.0 * m
     fwd_ms = (tm["prep_ms"] + tm["grid_ms"] + tm["fft_ms"] + tm["stack_ms"]) / max(tm["stack_calls"], 1)
     if rank == 0:
         print(json.dumps({
