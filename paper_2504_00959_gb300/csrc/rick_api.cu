@@ -201,8 +201,10 @@ bool use_split(const rick_params& p, int* n1, int* n2)
 // 1024, 2048, 4096 unless RICK_FFT_2D asks for cuFFT's 2D plan, and up to
 // kStripAmp.  Measured, with the split transform before it: 4096^2 x 32 planes
 // x 1e7 measurements 4.99 -> 3.52 ms per image, 8 channels of 2048^2 x 16
-// 5.70 -> 4.72 ms, 1024^2 x 16 x 1e6 0.358 -> 0.343 ms.  It needs a second buffer of a group's planes (strip order); where that does not fit,
-// the handle takes the split transform or the 2D plan instead.
+// 5.70 -> 4.08 ms, 1024^2 x 16 x 1e6 0.358 -> 0.301 ms (0.343 without the scan in
+// one launch and the gridder's smaller blocks).  It needs a second buffer of a
+// group's planes (strip order); where that would take more than half of the
+// free memory, the handle takes the split transform or the 2D plan instead.
 bool want_strip(const rick_params& p) { return strip_shape(p.n) && !(p.flags & RICK_FFT_2D); }
 
 // Grid correction multiplies the planes' rounding (~3e-7 of their RMS,
@@ -428,7 +430,9 @@ bool strip_alloc(rick_handle h, bool strip)
     const size_t tab = strip ? (size_t)h->nchan * (n / 2 + 1) * (n / 2 + 16) : 0;
     const size_t tab_bytes = 3 * tab * sizeof(float2), strip_bytes = strip ? (size_t)h->G * pb : 0;
     const size_t need = strip_bytes + bits + rng + tw + tab_bytes;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || need + (64u << 20) > fr) return false;
+    // at most half of what is free: the rest is for the sorted measurements,
+    // whose number is not known yet
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || 2 * need + (64u << 20) > fr) return false;
     std::vector<float2> w(tw / sizeof(float2));
     for (int k = 1; k < 16; ++k) {
         for (int j = 0; j < n / 16; ++j) {

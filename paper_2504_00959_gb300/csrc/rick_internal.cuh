@@ -376,7 +376,6 @@ cudaError_t launch_colimage(const StripArgs& s, const StackArgs& a, const float2
 cudaError_t launch_colspread(const StripArgs& s, const StackArgs& a, const void* rimg, const double* sum_w,
                              float2* strips, cudaStream_t st);
 
-// nchan > 1: channels a.chan0 .. of a batch in one launch (as launch_colstack)
 // ---- sparse rows of the split transform, n = 8192 and 16384 (rick_longrow.cu):
 // in place, bits / range / twiddles as above with tw1 w_n^(j k1) [15][n / 16],
 // tw2 w_(n/16)^(t2 k2) [15][n / 256], then w_(n/256)^(s k3) [15][n / 4096]
@@ -384,6 +383,7 @@ bool longrow_shape(int n);
 cudaError_t launch_longrows(int n, int dir, const StripArgs& s, int k0, int nk, int row_perm, float2* planes,
                             cudaStream_t st);
 
+// nchan > 1: channels a.chan0 .. of a batch in one launch (as launch_colstack)
 cudaError_t launch_stack(const StackArgs& a, const float2* planes, float2* acc, const float* taper,
                          const double* sum_w, void* image, cudaStream_t s, int nchan = 1);
 
