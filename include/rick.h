@@ -64,12 +64,11 @@ typedef int32_t rick_status;
                                   cover the folded range (w_min, w_max >= 0 typically: half the
                                   planes for the same plane spacing) */
 #define RICK_FFT_2D 64u         /* transform the planes with cuFFT's 2D plan and stack them in a
-                                  separate pass, also where the library would otherwise split
-                                  the column transform and fuse its last factor with the
-                                  w-screen and the stack (single images with n >= 2048) */
+                                  separate pass, also where the library would otherwise take
+                                  its own transforms (power-of-two n from 1024 to 16384) */
 #define RICK_FFT_SPLIT 128u     /* the split transform for any power-of-two n in [64, 16384]
-                                  (single images; the default from n = 2048 on, for tests and
-                                  measurement below).  Not with RICK_FFT_2D.  Either way the
+                                  where the library would otherwise take cuFFT's 2D plan
+                                  (single images; for tests and measurement).  Not with RICK_FFT_2D.  Either way the
                                   result is the same up to rounding */
 
 /* Problem statement of Sec. 2.1: grid size, pixel scale, w-planes, kernel.
@@ -158,14 +157,20 @@ rick_status rick_add_density(rick_handle h, const float* vis, const float* u, co
  * (cuFFT, unnormalised, exponent +), multiply by the phase screen
  * exp(+2 pi i w_k (n-1)) and sum over planes (Eq. 1); then divide by the
  * weight sum and, per flags, by the taper and times n.  image: float[n*n]
- * (RICK_REAL_IMAGE) or float[2*n*n] complex, fully overwritten.  For
- * power-of-two n from 2048 to 16384 (or with RICK_FFT_SPLIT) the column
- * transform is split, n = 16 * (n / 16): cuFFT transforms the rows, one
- * library kernel the first (n / 16-point) column factor of every plane of
- * the group in place, and one kernel the last 16-point column factor
- * together with the screen and the sum, reading each plane once more;
- * otherwise cuFFT's 2D plan and a separate screen-and-sum pass
- * (RICK_FFT_2D). */
+ * (RICK_REAL_IMAGE) or float[2*n*n] complex, fully overwritten.  For n =
+ * 1024, 2048 and 4096 two library kernels per plane group do the transform:
+ * one the rows, of the tiles that hold entries, into a second buffer of the
+ * group's planes, and one the whole column transform together with the
+ * screen and the sum, reading that buffer once.  For n = 8192 and 16384 (or
+ * with RICK_FFT_SPLIT) the column transform is split, n = 16 * (n / 16): the
+ * rows are transformed in place, one library kernel does the first (n / 16-
+ * point) column factor of every plane of the group in place, and one the
+ * last 16-point column factor together with the screen and the sum.
+ * Otherwise, and with RICK_FFT_2D, cuFFT's 2D plan and a separate
+ * screen-and-sum pass.  Where the second buffer would take more than half of
+ * the device memory that is free, and where the grid correction amplifies rounding by more
+ * than 300 (mean of 1 / taper^2; support 8 or a Gaussian of 6 and wider),
+ * n = 2048 and 4096 take the split and n = 1024 the 2D plan. */
 rick_status rick_fft_and_stack(rick_handle h, float* image);
 
 /* Eq. 3 alone: the gridded planes k0 .. k0+nk-1 as complex float
@@ -233,10 +238,10 @@ rick_status rick_synchronize(rick_handle h);
 rick_status rick_create_batch(const rick_params* p, int32_t nchan, const double* w_min, const double* w_max,
                               rick_handle* out);
 /* (Batched handles transform their plane groups like single images from
- * n = 1024 on -- cuFFT's rows, the library's first column factor, and one
- * launch of the last column factor fused with every channel's w-screen and
- * stack -- and with cuFFT's 2D plan and a separate stack per channel below,
- * or with RICK_FFT_2D.  Hermitian fold works per channel; each channel's
+ * n = 1024 on, one launch of each kernel for all channels of a group (n =
+ * 1024 too takes the split where the two kernels are not taken), and with
+ * cuFFT's 2D plan and one launch of the stack for the group's channels
+ * below, or with RICK_FFT_2D.  Hermitian fold works per channel; each channel's
  * w-range is then its folded one.) */
 
 /* One dirty image per channel: channel c's measurements are entries
@@ -334,9 +339,9 @@ rick_status rick_set_plane_range(rick_handle h, int32_t k0, int32_t k1);
  * for batched handles. */
 rick_status rick_set_weight_sum(rick_handle h, double sum_w);
 
-/* Test hook of the error path of the fused column-transform kernel (the
- * split transform of rick_fft_and_stack; the paper has no counterpart).
- * Every wait of that kernel on its shared-memory pipeline is bounded; with
+/* Test hook of the error path of the column-transform kernels fused with
+ * the stack (rick_fft_and_stack; the paper has no counterpart).
+ * Every wait of those kernels on their shared-memory pipeline is bounded; with
  * skip_slot >= 0 the kernel's producer leaves out the copy of that pipeline
  * slot (plane nk - 1 - skip_slot of a group of nk), so every thread block's
  * wait on it runs out after wait_ns nanoseconds (<= 0: the default 1 s), the
@@ -354,11 +359,12 @@ rick_status rick_get_stats(rick_handle h, rick_stats* out);
 
 /* Per-phase device time of the library's own work, from CUDA events recorded
  * on the handle's stream around each phase (no synchronisation while timing
- * is on).  Phases: prep = placement + counting sort (rick_grid); grid = the
- * gridding kernel (Eq. 3); fft = cuFFT plane transforms (the rows only when
- * the column transform is split); colfft = the first column factor of the
- * split transform (the library's own kernel); stack = phase screen + plane
- * reduction + finalisation (with the split: the last column factor too);
+ * is on).  Phases: prep = placement + counting sort (rick_grid) and
+ * the marking of the tiles that hold entries; grid = the gridding kernel
+ * (Eq. 3); fft = the row transforms (the 2D plan where cuFFT's is taken);
+ * colfft = the first column factor of the split transform; stack = phase
+ * screen + plane reduction + finalisation, with the library's own transforms
+ * fused with the column transform (n = 1024 to 4096) or its last factor;
  * degrid = the whole adjoint.  Times are sums over all calls since timing
  * was enabled; *_calls count the phase executions; kernel_launches counts
  * librick's own kernel launches (cuFFT's not included). */

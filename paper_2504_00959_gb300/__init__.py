@@ -2,7 +2,7 @@
 
 Python binding over the C ABI of ``librick.so`` (include/rick.h).  PyTorch is
 used for device memory and streams only; gridding (Eq. 3), the per-plane
-inverse FFT (cuFFT), the w-term phase-screen stack (Eq. 1) and the adjoint
+inverse FFT, the w-term phase-screen stack (Eq. 1) and the adjoint
 degridder all run in the library.  There is no CPU fallback: constructing an
 ``Imager`` without the built library, or with tensors that are not on a CUDA
 device, raises.
@@ -264,7 +264,7 @@ class Imager:
 
 class BatchImager(Imager):
     """Many frequency channels imaged together (one sort, one gridder pass and
-    one cuFFT batch per plane group, one stack per channel).  ``w_ranges`` is
+    one launch of each transform kernel and of the stack per plane group).  ``w_ranges`` is
     a sequence of (w_min, w_max) per channel; the other parameters are shared."""
 
     def __init__(self, params, w_ranges, device=None):
