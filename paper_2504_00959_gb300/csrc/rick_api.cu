@@ -1107,7 +1107,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
     size_t fr = 0, tot = 0;
     RICK_CU(h, cudaMemGetInfo(&fr, &tot));
     // the sorted measurements where they fit, else their indices
-    const bool by_rows = !(h->amp <= kGatherAmp);
+    const bool by_rows = !(h->amp <= kGatherAmp) || !gather_by_columns(c, nvis);
     const bool with_entries = !by_rows && off_bytes + primary_list_bytes(nvis, true) + (64u << 20) <= fr;
     const size_t perm_bytes = primary_list_bytes(nvis, with_entries);
     if (off_bytes + perm_bytes + (64u << 20) > fr) return fail(h, RICK_ERR_OOM, "degrid scratch does not fit");

@@ -401,6 +401,7 @@ cudaError_t launch_primary_scatter(const GridCfg& c, const float* u, const float
                                    void* list, bool with_entries, cudaStream_t s);
 // by_rows: one thread per measurement, the footprint summed row by row (a list
 // of indices)
+bool gather_by_columns(const GridCfg& c, int64_t m);
 cudaError_t launch_degrid_gather(const GridCfg& c, void* list, bool with_entries, bool by_rows, int64_t m,
                                  const uint32_t* offsets, int k0, int nk, const float2* planes, const float* u, const float* v, const float* w,
                                  const float* wt, const uint32_t* density, float2* grad, cudaStream_t s);

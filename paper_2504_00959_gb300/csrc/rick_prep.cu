@@ -354,11 +354,12 @@ PrimaryList primary_list(void* p, int64_t m, bool with_entries)
     return PrimaryList{ent, reinterpret_cast<int*>(ent + m), nullptr};
 }
 
-// Lanes that gather one measurement: one per footprint column.
+// Lanes that gather one measurement in k_degrid_gather: one per footprint
+// column (supports 4, 7 and 8: gather_by_columns).
 template <int S>
 __host__ __device__ constexpr int gather_lanes()
 {
-    return S <= 4 ? 4 : (S <= 8 ? 8 : 16);
+    return S <= 4 ? 4 : 8;
 }
 
 // Each sorted measurement of planes [k0, k0+nk) gathers its S x S footprint
@@ -500,9 +501,10 @@ __global__ void __launch_bounds__(kPrepThreads) k_degrid_gather(GridCfg c, Prima
 // Each sorted measurement of planes [k0, k0+nk) gathers its S x S footprint
 // of the (forward-transformed) adjoint planes with the gridding taps, times
 // its effective weight, one thread per measurement, the taps summed row by
-// row.  Only for kernels whose grid correction amplifies rounding (kGatherAmp):
+// row.  For kernels whose grid correction amplifies rounding (kGatherAmp):
 // there the sum of a footprint cancels to far below its terms, and another
-// order of summation is another result.
+// order of summation is another result; and where gather_by_columns measured
+// it the faster one.
 template <int S>
 __global__ void __launch_bounds__(kPrepThreads) k_degrid_gather_rows(GridCfg c, const uint32_t* __restrict__ perm,
                                                                      const uint32_t* __restrict__ off, int k0, int nk,
@@ -761,6 +763,20 @@ cudaError_t launch_gather_s(const GridCfg& c, const PrimaryList& list, const uin
     return cudaGetLastError();
 }
 
+// Whether k_degrid_gather (a lane per footprint column) is to gather m
+// measurements, and k_degrid_gather_rows otherwise: supports that fill its
+// groups of 4 or 8 lanes, and lists that fill the chip's warps, each of which
+// takes 32 measurements one group step after another.  Predictions, row by row
+// and by columns, us: support 8 at 2000^2 x 8 planes, 5e4 measurements 350 and 349, 3e5
+// 378 and 374, 6e6 973 and 861, at 512^2 5e4 71 and 79, 3e5 97 and 96, 6e6 771 and 681;
+// support 4 at 2000^2 6e6 785 and 693.  Lanes without a column cost what the
+// kernel gains: support 6 at 512^2, 3e5 85 and 100, 6e6 610 and 631; support 9 at
+// 2000^2 6e6 1069 and 1184; support 12 1403 and 1350 there, but 411 and 432 at 3e5.
+bool gather_by_columns(const GridCfg& c, int64_t m)
+{
+    return (c.S == 4 || c.S == 7 || c.S == 8) && m >= ((int64_t)1 << 18);
+}
+
 cudaError_t launch_degrid_gather(const GridCfg& c, void* list, bool with_entries, bool by_rows, int64_t m,
                                  const uint32_t* offsets, int k0, int nk, const float2* planes, const float* u, const float* v, const float* w,
                                  const float* wt, const uint32_t* density, float2* grad, cudaStream_t s)
@@ -769,11 +785,18 @@ cudaError_t launch_degrid_gather(const GridCfg& c, void* list, bool with_entries
     if (by_rows && with_entries) return cudaErrorInvalidValue;  // takes the indices
     const Inputs in{u, v, w, wt, nullptr};
     const PrimaryList pl = primary_list(list, m, with_entries);
+    if (!by_rows) {
+        switch (c.S) {
+            case 4: return launch_gather_s<4>(c, pl, offsets, k0, nk, planes, in, density, grad, m, s);
+            case 7: return launch_gather_s<7>(c, pl, offsets, k0, nk, planes, in, density, grad, m, s);
+            case 8: return launch_gather_s<8>(c, pl, offsets, k0, nk, planes, in, density, grad, m, s);
+            default: return cudaErrorInvalidValue;
+        }
+    }
     switch (c.S) {
 #define RICK_GATHER_CASE(SS) \
-    case SS:                                                                                          \
-        return by_rows ? launch_gather_rows_s<SS>(c, pl.perm, offsets, k0, nk, planes, in, density, grad, s) \
-                       : launch_gather_s<SS>(c, pl, offsets, k0, nk, planes, in, density, grad, m, s);
+    case SS:                       \
+        return launch_gather_rows_s<SS>(c, pl.perm, offsets, k0, nk, planes, in, density, grad, s);
         RICK_GATHER_CASE(1) RICK_GATHER_CASE(2) RICK_GATHER_CASE(3) RICK_GATHER_CASE(4)
         RICK_GATHER_CASE(5) RICK_GATHER_CASE(6) RICK_GATHER_CASE(7) RICK_GATHER_CASE(8)
         RICK_GATHER_CASE(9) RICK_GATHER_CASE(10) RICK_GATHER_CASE(11) RICK_GATHER_CASE(12)

@@ -1,6 +1,7 @@
-"""The adjoint's gather at every number of lanes per measurement (supports up
-to 4, 8 and 16), at footprints across tile edges and at the grid's edges, for
-lists shorter and longer than a warp's 32 measurements, against the FP64
+"""The adjoint's gather, row by row for short lists and most supports and a lane
+per footprint column for long lists of supports 4, 7 and 8 (at the first list
+length that takes it, and at one that leaves the last warp a single
+measurement), at footprints across tile edges and at the grid's edges, against the FP64
 oracle's adjoint at the bar of the other adjoint tests (1e-4 of the largest
 component); and the row-by-row gather that kernels with an amplifying grid
 correction keep, with the gradient of an image in the well-conditioned centre."""
@@ -45,6 +46,15 @@ def test_supports(rick, oracle_mod, S, m):
     prob = synth.disk_problem(128, 3, m, synth.KERNEL_KB, S, 4.0, 60.0, 700 + S + m, fill=0.55, weights="random")
     r = np.random.default_rng(S).standard_normal((128, 128)).astype(np.float32)
     _check(rick, oracle_mod, prob, REAL, r)
+
+
+@pytest.mark.parametrize("S", [4, 7, 8])
+@pytest.mark.parametrize("m,flags,extra", [(1 << 18, REAL, {}), ((1 << 18) + 33, REAL | synth.FLAG_UNIFORM, {"tile": 16}),
+                                           ((1 << 18) + 1, REAL, {"w_support": 3, "plane_group": 2, "tile": 64})])
+def test_columns(rick, oracle_mod, S, m, flags, extra):
+    prob = synth.disk_problem(130, 6, m, synth.KERNEL_KB, S, 4.0, 60.0, 760 + S, fill=0.55, weights="random")
+    r = np.random.default_rng(S).standard_normal((130, 130)).astype(np.float32)
+    _check(rick, oracle_mod, prob, flags, r, **extra)
 
 
 @pytest.mark.parametrize("flags,extra", [(REAL | synth.FLAG_UNIFORM, {"tile": 16}),
