@@ -664,9 +664,11 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_add(const uint32_t* __restr
 // cluster, each CTA a run of `per` counters (a multiple of kScanTile) in
 // registers; the CTAs exchange their totals through distributed shared memory.
 // The sort of 1e5 measurements into 512 tiles took 35 us with three launches
-// for the scan and takes 28 with one; 1e6 into 16384 tiles 85 and 78.
+// for the scan and takes 28 with one; 1e6 into 16384 tiles 85 and 78.  Eight
+// SMs fall behind beyond: 5e5 into 32768 tiles 53.5 and 47.8, into 65536 54.6 and
+// 54.3, into 105300 and 131072 54.8 and 65.
 constexpr int kScanCluster = 8;
-constexpr int kScanSub = 4;  // tiles of kScanTile counters per CTA at most
+constexpr int kScanSub = 2;  // tiles of kScanTile counters per CTA at most
 constexpr int64_t kScanMax = (int64_t)kScanCluster * kScanSub * kScanTile;
 
 __global__ void __cluster_dims__(kScanCluster, 1, 1) __launch_bounds__(kScanBlock)

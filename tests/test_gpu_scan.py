@@ -12,7 +12,7 @@ import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nw", [1, 255, 256, 257, 2048, 2049, 8192, 8193])
+@pytest.mark.parametrize("nw", [1, 255, 256, 257, 2048, 2049, 4096, 4097, 8192, 8193])
 def test_plane_sums(nw):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
