@@ -366,7 +366,7 @@ rick_status colfft_ready(rick_handle h)
         h->bytes_held += sizeof(float2) * n1;
     }
     RICK_CU(h, cudaMemcpy(h->cf_tw, tw.data(), sizeof(float2) * n1, cudaMemcpyHostToDevice));
-    RICK_CU(h, encode_colfft_map(h->cfmap, h->planes, h->p.n, h->G));
+    RICK_CU(h, encode_colfft_map(h->cfmap, h->planes, h->p.n, h->G, h->longrows));
     h->cfmap_ready = true;
     return RICK_OK;
 }
@@ -844,7 +844,7 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
         if (encode_colstack_map(h->colmap, h->planes, p->n, h->G) != cudaSuccess) return cleanup(RICK_ERR_CUDA);
         h->colmap_ready = true;
         if (h->planes2 && (encode_colstack_map(h->colmap2, h->planes2, p->n, h->G) != cudaSuccess ||
-                           encode_colfft_map(h->cfmap2, h->planes2, p->n, h->G) != cudaSuccess))
+                           encode_colfft_map(h->cfmap2, h->planes2, p->n, h->G, h->longrows) != cudaSuccess))
             return cleanup(RICK_ERR_CUDA);
     }
     if (cudaDeviceSynchronize() != cudaSuccess) return cleanup(RICK_ERR_CUDA);

@@ -45,7 +45,9 @@ namespace {
 
 constexpr int kCfThreads = 256;
 constexpr unsigned long long kCfWaitNs = 1000000000ull;  // bound of the load wait: 1 s
-constexpr int kCfBoxRows = 128;  // TMA box: rows per copy (the unit in which empty rows are left out)
+// TMA box: rows per copy at most; with row ranges they are the unit in which
+// empty rows are left out
+constexpr int kCfBoxRows = 256, kCfRangeBoxRows = 128;
 
 __device__ __forceinline__ float2 c_add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 c_sub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
@@ -264,18 +266,18 @@ __device__ __forceinline__ void colfft_two_pass(float2* __restrict__ buf, const 
 // memory N1 * W complex values, the N1 twiddles and one mbarrier.  tw:
 // exp(+2 pi i j / N1), j < N1 (device; copied in with the block's data).
 // err: bit 1 set when the load wait ran out.
-// range (or NULL: all): the tile rows [lo, hi) of each plane that hold anything
+// range (RANGE; else all): the tile rows [lo, hi) of each plane that hold anything
 // (imaging: the other rows are taken as zeros and not read) or are wanted
 // (adjoint: the other rows are not written); tile sides are multiples of 16,
 // so the rows 16 a + b of every b have the same range of a.
-template <int N1, int W, int SIGN>
+template <int N1, int W, int SIGN, bool RANGE>
 __global__ void __launch_bounds__(kCfThreads) k_colfft(const __grid_constant__ CUtensorMap map,
                                                        const float2* __restrict__ tw, float2* __restrict__ planes,
                                                        int n, const int2* __restrict__ range, int log2T,
                                                        unsigned long long wait_ns,
                                                        unsigned long long* __restrict__ err)
 {
-    constexpr int kBox = N1 < kCfBoxRows ? N1 : kCfBoxRows;
+    constexpr int kRows = RANGE ? kCfRangeBoxRows : kCfBoxRows, kBox = N1 < kRows ? N1 : kRows;
     extern __shared__ __align__(128) unsigned char cf_smem[];
     float2* buf = reinterpret_cast<float2*>(cf_smem);  // [N1][W]
     float2* tws = buf + (size_t)N1 * W;                 // [N1] twiddles
@@ -286,7 +288,7 @@ __global__ void __launch_bounds__(kCfThreads) k_colfft(const __grid_constant__ C
     const int x0 = blockIdx.x * W, b = blockIdx.y, plane = blockIdx.z;
     const unsigned long long limit = wait_ns ? wait_ns : kCfWaitNs;
     int alo = 0, ahi = N1;
-    if (range) {
+    if (RANGE) {
         const int2 rg = __ldg(range + plane);
         alo = (rg.x << log2T) >> 4;
         ahi = (rg.y << log2T) >> 4;
@@ -339,7 +341,7 @@ __global__ void __launch_bounds__(kCfThreads) k_colfft(const __grid_constant__ C
     }
 }
 
-template <int N1, int W, int SIGN>
+template <int N1, int W, int SIGN, bool RANGE>
 cudaError_t launch_cf(const void* map, const float2* tw, float2* planes, int n, int nk, const int2* range, int log2T,
                       unsigned long long wait_ns, unsigned long long* err, cudaStream_t s)
 {
@@ -349,12 +351,12 @@ cudaError_t launch_cf(const void* map, const float2* tw, float2* planes, int n, 
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_done[dev]) {
         const cudaError_t e =
-            cudaFuncSetAttribute(k_colfft<N1, W, SIGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaFuncSetAttribute(k_colfft<N1, W, SIGN, RANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr_done[dev] = true;
     }
     const dim3 grid((unsigned)(n / W), 16u, (unsigned)nk);
-    k_colfft<N1, W, SIGN><<<grid, kCfThreads, smem, s>>>(*reinterpret_cast<const CUtensorMap*>(map), tw, planes,
+    k_colfft<N1, W, SIGN, RANGE><<<grid, kCfThreads, smem, s>>>(*reinterpret_cast<const CUtensorMap*>(map), tw, planes,
                                                           n, range, log2T, wait_ns, err);
     return cudaGetLastError();
 }
@@ -374,7 +376,7 @@ int colfft_width(int n1)
     return n1 <= 256 ? 16 : 8;
 }
 
-cudaError_t encode_colfft_map(void* map, const float2* planes, int n, int planes_in_buffer)
+cudaError_t encode_colfft_map(void* map, const float2* planes, int n, int planes_in_buffer, bool ranges)
 {
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     if (!encode) {
@@ -391,7 +393,8 @@ cudaError_t encode_colfft_map(void* map, const float2* planes, int n, int planes
     // row 16 a + b of plane p (memory row b N1 + a) is (a, 16 p + b)
     const cuuint64_t dims[3] = {(cuuint64_t)n, (cuuint64_t)n1, (cuuint64_t)planes_in_buffer * 16};
     const cuuint64_t strides[2] = {(cuuint64_t)n * sizeof(float2), (cuuint64_t)n1 * n * sizeof(float2)};
-    const cuuint32_t box[3] = {(cuuint32_t)w, (cuuint32_t)(n1 < kCfBoxRows ? n1 : kCfBoxRows), 1};
+    const int rows = ranges ? kCfRangeBoxRows : kCfBoxRows;
+    const cuuint32_t box[3] = {(cuuint32_t)w, (cuuint32_t)(n1 < rows ? n1 : rows), 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = encode(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_UINT64, 3,
                               const_cast<float2*>(planes), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -408,9 +411,18 @@ cudaError_t launch_colfft(const void* map, const float2* tw, float2* planes, int
     const int n1 = n / 16;
 #define RICK_CF_CASE(N1)                                                                                   \
     case N1:                                                                                               \
-        return sign > 0 ? launch_cf<N1, cf_width<N1>(), 1>(map, tw, planes, n, nk, range, log2T, wait_ns, err, s)        \
-                        : launch_cf<N1, cf_width<N1>(), -1>(map, tw, planes, n, nk, range, log2T, wait_ns, err, s);
-    if (n != 16 * n1 || (range && n1 < 16)) return cudaErrorInvalidValue;
+        return sign > 0 ? launch_cf<N1, cf_width<N1>(), 1, RANGE>(map, tw, planes, n, nk, range, log2T, wait_ns, err, s) \
+                        : launch_cf<N1, cf_width<N1>(), -1, RANGE>(map, tw, planes, n, nk, range, log2T, wait_ns, err, s);
+    if (n != 16 * n1) return cudaErrorInvalidValue;
+    if (range) {  // of the planes of k_longrows
+        constexpr bool RANGE = true;
+        switch (n1) {
+            RICK_CF_CASE(512)
+            RICK_CF_CASE(1024)
+            default: return cudaErrorInvalidValue;
+        }
+    }
+    constexpr bool RANGE = false;
     switch (n1) {
         RICK_CF_CASE(4)
         RICK_CF_CASE(8)

@@ -329,7 +329,7 @@ cudaError_t launch_colstack(const void* map, const StackArgs& a, int n1, int n2,
 // (k_colfft, rick_colfft.cu): rows 16 a + b -> rows 16 f1 + b in place, the
 // N1 = n / 16-point DFT with exponent sign (+1 imaging, -1 adjoint); map
 // from encode_colfft_map for the plane buffer, tw = exp(+2 pi i j / N1)
-cudaError_t encode_colfft_map(void* map, const float2* planes, int n, int planes_in_buffer);
+cudaError_t encode_colfft_map(void* map, const float2* planes, int n, int planes_in_buffer, bool ranges);
 // range (of the group's planes; NULL: all rows): see k_colfft
 cudaError_t launch_colfft(const void* map, const float2* tw, float2* planes, int n, int nk, int sign,
                           const int2* range, int log2T, unsigned long long wait_ns, unsigned long long* err, cudaStream_t s);
