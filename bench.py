@@ -830,8 +830,7 @@ def run_channels(args, rank, world):
         return f0.elapsed_time(f1) / ksteps, k0, k1
 
     # the per-channel loop with the library's default single-image path, and
-    # with RICK_FFT_SPLIT (which only sizes outside 1024 .. 4096 tell apart);
-    # the faster one is the reference
+    # with RICK_FFT_SPLIT; the faster one is the reference
     t_loop, k0, k1 = time_loop()
     loop_default = loop_out.clone()
     for im in ims:

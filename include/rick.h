@@ -66,10 +66,12 @@ typedef int32_t rick_status;
 #define RICK_FFT_2D 64u         /* transform the planes with cuFFT's 2D plan and stack them in a
                                   separate pass, also where the library would otherwise take
                                   its own transforms (power-of-two n from 1024 to 16384) */
-#define RICK_FFT_SPLIT 128u     /* the split transform for any power-of-two n in [64, 16384]
-                                  where the library would otherwise take cuFFT's 2D plan
-                                  (single images; for tests and measurement).  Not with RICK_FFT_2D.  Either way the
-                                  result is the same up to rounding */
+#define RICK_FFT_SPLIT 128u     /* the split transform with cuFFT's rows for any power-of-two n in
+                                  [64, 16384] (batched handles: from n = 1024), also where the
+                                  library would otherwise take its two kernels over what is not
+                                  empty (n = 1024 to 4096, which hold a second plane buffer) or
+                                  its sparse rows (n = 8192, 16384).  Not with RICK_FFT_2D.
+                                  Either way the result is the same up to rounding */
 
 /* Problem statement of Sec. 2.1: grid size, pixel scale, w-planes, kernel.
  * n: grid side, even, >= 2*support.  nw >= 1.  w_max > w_min when nw > 1.
@@ -162,8 +164,8 @@ rick_status rick_add_density(rick_handle h, const float* vis, const float* u, co
  * one the rows, of the tiles that hold entries, into a second buffer of the
  * group's planes, and one the whole column transform together with the
  * screen and the sum, reading that buffer once.  For n = 8192 and 16384 (or
- * with RICK_FFT_SPLIT) the column transform is split, n = 16 * (n / 16): the
- * rows are transformed in place, one library kernel does the first (n / 16-
+ * with RICK_FFT_SPLIT, then with cuFFT's rows) the column transform is split,
+ * n = 16 * (n / 16): the rows are transformed in place, one library kernel does the first (n / 16-
  * point) column factor of every plane of the group in place, and one the
  * last 16-point column factor together with the screen and the sum.
  * Otherwise, and with RICK_FFT_2D, cuFFT's 2D plan and a separate

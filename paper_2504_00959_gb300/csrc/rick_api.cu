@@ -198,14 +198,15 @@ bool use_split(const rick_params& p, int* n1, int* n2)
 
 // The two-pass transform of rick_strip.cu (row transforms of what is not empty,
 // then the whole column transform fused with the screen and the stack): n =
-// 1024, 2048, 4096 unless RICK_FFT_2D asks for cuFFT's 2D plan, and up to
-// kStripAmp.  Measured, with the split transform before it: 4096^2 x 32 planes
+// 1024, 2048, 4096 unless RICK_FFT_2D or RICK_FFT_SPLIT asks for another one, and
+// up to kStripAmp.  Measured, with the split transform before it: 4096^2 x 32 planes
 // x 1e7 measurements 4.99 -> 3.52 ms per image, 8 channels of 2048^2 x 16
 // 5.70 -> 4.08 ms, 1024^2 x 16 x 1e6 0.358 -> 0.301 ms (0.343 without the scan in
 // one launch and the gridder's smaller blocks).  It needs a second buffer of a
 // group's planes (strip order); where that would take more than half of the
 // free memory, the handle takes the split transform or the 2D plan instead.
-bool want_strip(const rick_params& p) { return strip_shape(p.n) && !(p.flags & RICK_FFT_2D); }
+bool own_transform(const rick_params& p) { return !(p.flags & (RICK_FFT_2D | RICK_FFT_SPLIT)); }
+bool want_strip(const rick_params& p) { return strip_shape(p.n) && own_transform(p); }
 
 // Grid correction multiplies the planes' rounding (~3e-7 of their RMS,
 // uncorrelated between pixels) by 1 / (c(x) c(y)), over the image by mean(1 /
@@ -223,7 +224,7 @@ constexpr double kStripAmp = 300.0;
 // 47.5 -> 41.4 ms (gridding 6.8 -> 4.9, rows 18.3 -> 13.6), 8192^2 x 4 x 3e4 2.76
 // -> 2.40 ms.
 constexpr double kLongAmp = 600.0;
-bool want_longrows(const rick_params& p) { return longrow_shape(p.n) && !(p.flags & RICK_FFT_2D); }
+bool want_longrows(const rick_params& p) { return longrow_shape(p.n) && own_transform(p); }
 // The adjoint's footprints, of planes that hold the corrected image, cancel by
 // the same factors: where they cancel by more than binary32 holds, the gather
 // keeps its order of summation too.
