@@ -346,6 +346,19 @@ rick_status check_vis_args(rick_handle h, const float* vis, const float* u, cons
     return RICK_OK;
 }
 
+// What the handle's pool holds and no allocation uses: the pool keeps what is
+// freed to it, which cudaMemGetInfo therefore does not count as free.
+size_t pool_idle(rick_handle h)
+{
+    uint64_t held = 0, used = 0;
+    if (cudaMemPoolGetAttribute(h->pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+        cudaMemPoolGetAttribute(h->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return held > used ? (size_t)(held - used) : 0;
+}
+
 // The weight sum images are normalised by: the caller's (rick_set_weight_sum)
 // or the handle's own (device).
 const double* norm_sum(rick_handle h) { return h->sw_given ? h->sw_dev : &h->ctr->sum_w; }
@@ -1107,17 +1120,24 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
     const size_t off_bytes = (size_t)(ntiles + 1) * sizeof(uint32_t);
     size_t fr = 0, tot = 0;
     RICK_CU(h, cudaMemGetInfo(&fr, &tot));
+    fr += pool_idle(h);  // this call's scratch takes again what an earlier one's left in the pool
     // the sorted measurements where they fit, else their indices
     const bool by_rows = !(h->amp <= kGatherAmp) || !gather_by_columns(c, nvis);
-    const bool with_entries = !by_rows && off_bytes + primary_list_bytes(nvis, true) + (64u << 20) <= fr;
-    const size_t perm_bytes = primary_list_bytes(nvis, with_entries);
-    if (off_bytes + perm_bytes + (64u << 20) > fr) return fail(h, RICK_ERR_OOM, "degrid scratch does not fit");
+    bool with_entries = !by_rows && off_bytes + primary_list_bytes(nvis, true) + (64u << 20) <= fr;
+    if (off_bytes + primary_list_bytes(nvis, with_entries) + (64u << 20) > fr)
+        return fail(h, RICK_ERR_OOM, "degrid scratch does not fit");
     PhaseScope scope(h, kPhaseDegrid);
     uint32_t* off = nullptr;
     void* perm = nullptr;
     RICK_CU(h, cudaMallocFromPoolAsync((void**)&off, off_bytes, h->pool, h->stream));
-    cudaError_t e = cudaMallocFromPoolAsync(&perm, perm_bytes, h->pool, h->stream);
+    cudaError_t e = cudaMallocFromPoolAsync(&perm, primary_list_bytes(nvis, with_entries), h->pool, h->stream);
+    if (e != cudaSuccess && with_entries) {  // what is idle may be in pieces: the indices take less
+        (void)cudaGetLastError();
+        with_entries = false;
+        e = cudaMallocFromPoolAsync(&perm, primary_list_bytes(nvis, with_entries), h->pool, h->stream);
+    }
     if (e != cudaSuccess) {
+        (void)cudaGetLastError();  // reported here: the next launch's check does not find it
         cudaFreeAsync(off, h->stream);
         return fail(h, RICK_ERR_OOM, "cudaMallocFromPoolAsync(perm): %s", cudaGetErrorString(e));
     }
