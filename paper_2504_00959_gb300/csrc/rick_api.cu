@@ -424,10 +424,15 @@ void strip_free(rick_handle h)
     cudaFree(h->sargs.bits);
     cudaFree(h->sargs.range);
     cudaFree(h->sargs.tab.rho);
+    cudaFree(h->sargs.part);
     cudaFree(const_cast<float2*>(h->sargs.tw1));
     h->strips = nullptr;
     h->sargs = StripArgs{};
 }
+
+// The screen tables of a channel of nw planes: runs, and bytes (rho and one fin per run).
+int screen_runs(int nw) { return (nw + kScreenRun - 1) / kScreenRun; }
+size_t screen_bytes(int n, int runs) { return (size_t)(1 + runs) * (n / 2 + 1) * (n / 2 + 16) * sizeof(float2); }
 
 // Buffers and twiddles of the strip transform, or of the split transform's
 // sparse rows (rick_create); false where they do not fit.
@@ -440,10 +445,10 @@ bool strip_alloc(rick_handle h, bool strip)
     const size_t bits = (size_t)c.nw * c.ntu * wpr * sizeof(uint32_t), rng = (size_t)c.nw * sizeof(int2);
     const int q = strip ? 0 : n / 4096;
     const size_t t1 = 15 * (size_t)(n / 16), t2 = 15 * (size_t)r, tw = (t1 + t2 + 15 * (size_t)q) * sizeof(float2);
-    // entries of each screen table
-    const size_t tab = strip ? (size_t)h->nchan * (n / 2 + 1) * (n / 2 + 16) : 0;
-    const size_t tab_bytes = 3 * tab * sizeof(float2), strip_bytes = strip ? (size_t)h->G * pb : 0;
-    const size_t need = strip_bytes + bits + rng + tw + tab_bytes;
+    const int runs = screen_runs(c.nw_chan);
+    const size_t tab_bytes = strip ? h->nchan * screen_bytes(n, runs) : 0, strip_bytes = strip ? (size_t)h->G * pb : 0;
+    const size_t part_bytes = strip ? strip_part_bytes(runs) : 0;
+    const size_t need = strip_bytes + bits + rng + tw + tab_bytes + part_bytes;
     // at most half of what is free: the rest is for the sorted measurements,
     // whose number is not known yet
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || 2 * need + (64u << 20) > fr) return false;
@@ -467,19 +472,19 @@ bool strip_alloc(rick_handle h, bool strip)
               cudaMalloc((void**)&h->sargs.bits, bits) == cudaSuccess &&
               cudaMalloc((void**)&h->sargs.range, rng) == cudaSuccess &&
               (!strip || cudaMalloc((void**)&h->sargs.tab.rho, tab_bytes) == cudaSuccess) &&
+              (!part_bytes || cudaMalloc((void**)&h->sargs.part, part_bytes) == cudaSuccess) &&
               cudaMalloc((void**)&dev_tw, tw) == cudaSuccess;
     h->sargs.tw1 = dev_tw;
     h->sargs.tw2 = dev_tw ? dev_tw + t1 : nullptr;
     ok = ok && cudaMemcpy(dev_tw, w.data(), tw, cudaMemcpyHostToDevice) == cudaSuccess;
     if (ok && strip) {
-        h->sargs.tab.kap = h->sargs.tab.rho + tab;
-        h->sargs.tab.fin = h->sargs.tab.kap + tab;
+        h->sargs.tab.fin = h->sargs.tab.rho + (size_t)h->nchan * (n / 2 + 1) * (n / 2 + 16);
+        h->sargs.tab.runs = runs;
         ok = encode_rows_map(h->rowsmap, h->strips, n, h->G) == cudaSuccess;
         h->sargs.map = h->rowsmap;
         StackArgs a = stack_args(h);
         if (h->batch) a.chan_screen = h->chan_scr;
-        h->screen_k0 = 0;
-        ok = ok && launch_screen(h->sargs, a, h->taper, true, h->nchan, nullptr) == cudaSuccess;
+        ok = ok && launch_screen(h->sargs, a, h->taper, h->nchan, nullptr) == cudaSuccess;
     }
     if (!ok) {
         (void)cudaGetLastError();
@@ -490,18 +495,6 @@ bool strip_alloc(rick_handle h, bool strip)
     h->sargs.log2T = c.log2T;
     h->bytes_held += need;
     return true;
-}
-
-// The screen tables of a group whose first plane is k0.
-rick_status strip_screen(rick_handle h, const StackArgs& a, int k0)
-{
-    if (h->screen_k0 == k0) return RICK_OK;
-    StackArgs b = a;
-    b.k0 = k0;
-    RICK_CU(h, launch_screen(h->sargs, b, h->taper, false, 1, h->stream));
-    h->screen_k0 = k0;
-    count_launches(h, 1);
-    return RICK_OK;
 }
 
 // Grid planes [k0, k0 + nk) of every stored chunk into `planes`: the
@@ -601,7 +594,8 @@ rick_status rick_workspace_size(const rick_params* p, int64_t max_vis, size_t* b
     if (p->flags & RICK_UNIFORM_WEIGHT) b += (size_t)c.n * c.n * sizeof(uint32_t);
     if (want_strip(*p))  // the strip order's copy of a group, tile bits, row ranges, twiddles, screen
         b += (size_t)G * plane_bytes(p) + (size_t)c.nw * (c.ntu * ((c.ntu + 31) / 32) + 2) * sizeof(uint32_t) +
-             ((size_t)15 * (c.n / 16 + c.n / 256) + 3 * (size_t)(c.n / 2 + 1) * (c.n / 2 + 16)) * sizeof(float2);
+             (size_t)15 * (c.n / 16 + c.n / 256) * sizeof(float2) + screen_bytes(c.n, screen_runs(c.nw)) +
+             (c.nw > kScreenRun ? (size_t)160 * 512 * 16 * sizeof(float2) : 0);  // partial sums of at most 160 SMs
     b += plane_bytes(p);                                             // cuFFT work area (estimate)
     *bytes = b;
     return RICK_OK;
@@ -1063,7 +1057,6 @@ rick_status rick_fft_and_stack(rick_handle h, float* image)
                 count_launches(h, 1);
             }
             PhaseScope ss(h, kPhaseStack);
-            if ((s = strip_screen(h, a, k0))) return s;
             RICK_CU(h, launch_colimage(sa, a, h->strips, h->acc, norm_sum(h), image, &h->ctr->err, h->stream));
         } else if (split) {
             if ((s = colfft_ready(h))) return s;
@@ -1175,7 +1168,6 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
         a.nk = nk;
         if (h->strip) {
             sa.k0 = k0;
-            if ((st = strip_screen(h, a, k0))) break;
             e = launch_colspread(sa, a, image_grad, sum_w, h->strips, h->stream);
             if (e == cudaSuccess)
                 e = launch_rows(p.n, -1, sa, k0, nk, h->planes, h->dbg_wait_ns, &h->ctr->err, h->stream);

@@ -337,16 +337,20 @@ cudaError_t launch_spreadcol(const StackArgs& a, int n1, int n2, const void* rim
                              const double* sum_w, float2* planes, cudaStream_t s);
 
 // ---- the two-pass transform of n = 1024, 2048, 4096 (rick_strip.cu)
-// The w-screen of the pixels (k_screen): [nchan][n / 2 + 1][n / 2 + 16] each.
+// planes of a channel summed by Horner's rule between direct evaluations of the
+// screen: runs [32 r, 32 r + 32)
+constexpr int kScreenRun = 32;
+// The w-screen of the pixels (k_screen), tables of [n / 2 + 1][n / 2 + 16].
 struct ScreenTab {
-    float2* rho;  // rotation between planes
-    float2* kap;  // its correction over 32 planes
-    float2* fin;  // screen of the group's first plane times the finalisation
+    float2* rho;  // [nchan]: rotation between planes
+    float2* fin;  // [nchan][runs]: screen of the run's first plane times the finalisation
+    int runs;     // of a channel: ceil(nw / kScreenRun)
 };
 // What the kernels share: tile bits (wpr words per tile row) and non-empty
 // tile-row ranges of all planes of the handle (k_occupancy), the first plane
-// of the group that is in the strip buffer, and the twiddles w_n^(j k1)
-// ([15][n / 16], k1 = 1 .. 15) and w_(n/16)^(t2 k2) ([15][n / 256]).
+// of the group that is in the strip buffer, the twiddles w_n^(j k1)
+// ([15][n / 16], k1 = 1 .. 15) and w_(n/16)^(t2 k2) ([15][n / 256]), and the
+// partial sums of k_colimage's blocks between runs (strip_part_bytes).
 struct StripArgs {
     uint32_t* bits;
     int2* range;
@@ -354,6 +358,7 @@ struct StripArgs {
     const float2* tw1;
     const float2* tw2;
     ScreenTab tab;
+    float2* part;
     const void* map;  // tensor map of the strip buffer (encode_rows_map)
 };
 cudaError_t encode_rows_map(void* map, const float2* strips, int n, int planes);
@@ -362,10 +367,9 @@ bool strip_shape(int n);
 // reach > 0: tiles that the footprints of an adjoint sort (one list) touch,
 // w-footprints of `reach` planes
 cudaError_t launch_occupancy(const GridCfg& c, const ChunkList& ch, int reach, const StripArgs& s, cudaStream_t st);
-// the screen tables of nchan channels (chan_screen) or of the single image,
-// fin for the first plane a.k0; rho and kap only when with_rho
-cudaError_t launch_screen(const StripArgs& s, const StackArgs& a, const float* taper, bool with_rho, int nchan,
-                          cudaStream_t st);
+// the screen tables of nchan channels (chan_screen) or of the single image
+cudaError_t launch_screen(const StripArgs& s, const StackArgs& a, const float* taper, int nchan, cudaStream_t st);
+size_t strip_part_bytes(int runs);
 // dir +1: natural rows of planes [k0, k0 + nk) -> strips; -1: strips -> the needed tiles of the natural rows
 cudaError_t launch_rows(int n, int dir, const StripArgs& s, int k0, int nk, float2* planes,
                         unsigned long long wait_ns, unsigned long long* err, cudaStream_t st);
@@ -466,7 +470,6 @@ struct rick_imager {
     bool strip;
     float2* strips;                  // [G][n / 2][n] pairs of columns
     rick::StripArgs sargs;
-    int screen_k0;                   // the first plane sargs.tab.fin is for
     alignas(64) unsigned char rowsmap[128];  // tensor map of `strips` for k_rows
     float2* cf_tw;                   // [n / 16] exp(+2 pi i j / (n / 16)) for k_colfft
     struct Chunk {

@@ -383,25 +383,29 @@ constexpr size_t rows_smem()
 // ------------------------------------------------------- the pixels' screen
 
 // Per pixel, with n - 1 of the pixel: the rotation between planes rho = exp(2
-// pi i dw (n - 1)); kap = exp(2 pi i 32 dw (n - 1)) / rho^32, what products of
-// the binary32 rho miss over 32 planes; and fin = exp(2 pi i w_k0 (n - 1)) times
-// the finalisation's factors that do not depend on the data (taper, n and w
-// correction per flags, 0 outside the sky).  They depend on |x - n / 2| and |y -
-// n / 2| only and are symmetric in the two: one quadrant [a][b], a, b <= n / 2,
-// is kept, and the column kernels bring in the rows of their columns' a.  A
-// handle makes them once (fin again when k0 changes): evaluated per pixel
-// inside the column kernel, on 8 to 16 warps per SM, they took as long as 16
-// of its planes.  Entry b is stored at b ^ (b / 16 % 16): lanes whose pixels
-// are 16 rows apart then read 16 different banks.
+// pi i dw (n - 1)), and for every run of kScreenRun planes fin = exp(2 pi i w_k
+// (n - 1)) of the run's first plane k, times the finalisation's factors that do
+// not depend on the data (taper, n and w correction per flags, 0 outside the
+// sky).  Within a run the screen is a power of the binary32 rho; fin is
+// evaluated directly, so that what the powers miss does not add up from run to
+// run (RMS error of a sum of random planes over its RMS: 4e-7 for one run and
+// for 64; with a binary32 correction per run in its place 1e-6 at 4 runs, 2e-5
+// at 64).  The tables depend on |x - n / 2| and |y - n / 2| only and are
+// symmetric in the two: one quadrant [a][b], a, b <= n / 2, is kept, and the
+// column kernels bring in the rows of their columns' a.  A handle makes them
+// once: evaluated per pixel inside the column kernel, on 8 to 16 warps per SM,
+// they took as long as 16 of its planes.  Entry b is stored at b ^ (b / 16 %
+// 16): lanes whose pixels are 16 rows apart then read 16 different banks.
 __host__ __device__ __forceinline__ int screen_pitch(int n) { return n / 2 + 16; }
 __device__ __forceinline__ int screen_at(int b) { return b ^ ((b >> 4) & 15); }
 
-__global__ void __launch_bounds__(256) k_screen(StackArgs a_in, const float* __restrict__ taper, ScreenTab tab,
-                                                int with_rho)
+// grid z: run of a channel (tab.runs each)
+__global__ void __launch_bounds__(256) k_screen(StackArgs a_in, const float* __restrict__ taper, ScreenTab tab)
 {
     StackArgs a = a_in;
+    const int chan = (int)blockIdx.z / tab.runs, run = (int)blockIdx.z - chan * tab.runs;
     if (a_in.chan_screen) {
-        const float4 cs = __ldg(a_in.chan_screen + blockIdx.z);
+        const float4 cs = __ldg(a_in.chan_screen + chan);
         a.wb_hi = cs.x;
         a.wb_lo = cs.y;
         a.dw_hi = cs.z;
@@ -412,27 +416,17 @@ __global__ void __launch_bounds__(256) k_screen(StackArgs a_in, const float* __r
     if (ib > hn) return;
     const int x = hn - ia, y = hn - ib;  // pixels 0 .. n / 2
     const PixelScreen ps = pixel_screen(a, x, y);
-    const size_t at = ((size_t)blockIdx.z * (hn + 1) + ia) * pitch + screen_at(ib);
-    if (with_rho) {
-        const float2 rho = turns_to_phasor(ps.B.hi, ps.B.lo);
-        tab.rho[at] = rho;
-        const float2 e = turns_to_phasor(32.0f * ps.B.hi, 32.0f * ps.B.lo);
-        float2 p = rho;
-        for (int q = 0; q < 5; ++q) p = c_mul(p, p);
-        const float inv = 1.0f / (p.x * p.x + p.y * p.y);
-        tab.kap[at] = make_float2((e.x * p.x + e.y * p.y) * inv, (e.y * p.x - e.x * p.y) * inv);
-    }
+    if (run == 0)
+        tab.rho[((size_t)chan * (hn + 1) + ia) * pitch + screen_at(ib)] = turns_to_phasor(ps.B.hi, ps.B.lo);
     float f = ps.sky ? 1.0f : 0.0f;
     if (a.flags & RICK_GRID_CORRECT) f = f / (__ldg(taper + x) * __ldg(taper + y));
     if (a.flags & RICK_APPLY_N) f *= 1.0f + ps.nm1;
     if (a.wcorr) f /= wcorr_at(a, ps.nm1);
-    const float2 z = screen(ps.A, ps.B, a.k0);
-    tab.fin[at] = make_float2(z.x * f, z.y * f);
+    const float2 z = screen(ps.A, ps.B, run * kScreenRun);
+    tab.fin[((size_t)blockIdx.z * (hn + 1) + ia) * pitch + screen_at(ib)] = make_float2(z.x * f, z.y * f);
 }
 
 // ---------------------------------------------------------------- columns
-
-constexpr int kStripResync = 32;  // planes between corrections of the rotation (kap)
 
 // Blocks of the column kernels: kStrips strips of 2 x N / 16 threads; a thread
 // holds 16 positions of one column, and the Horner sum and the rotation of 16
@@ -512,23 +506,26 @@ struct ColThread {
     }
 };
 
-// the row of a screen table (all channels) of column x of a channel
+// the row of column x in table `t` (channel, or channel and run) of a ScreenTab member
 template <int N>
-__device__ __forceinline__ size_t screen_row(int chan, int x)
+__device__ __forceinline__ size_t screen_row(int t, int x)
 {
     const int d = x - N / 2;
-    return ((size_t)chan * (N / 2 + 1) + (d < 0 ? -d : d)) * screen_pitch(N);
+    return ((size_t)t * (N / 2 + 1) + (d < 0 ? -d : d)) * screen_pitch(N);
 }
 
 // Persistent blocks (as many as are co-resident) over the units of a launch:
 // a unit is kStrips strips of one channel, its slots are the rho rows of its
-// columns, the planes from the last to the first, and the fin rows.  The
+// columns, then the planes from the last to the first, and after each run's
+// first plane (and the unit's) the run's fin rows.  The
 // slots of consecutive units follow one another through three shared-memory
 // stages (bulk copies completing on the stage's mbarrier), so that a unit's
 // first copies are in flight while the last planes of the one before are
 // transformed.  Every slot has one block barrier, at which all threads are
 // done with the slot before: the copy of the slot two further on is issued
-// there.  Planes are summed per pixel by Horner's rule, h <- h rho + v.
+// there.  The planes of a run are summed per pixel by Horner's rule, h <- h rho +
+// v, and the runs' sums, times their fin, in `part` (a unit of one run does
+// without it; 64 KB per SM, which stay in L2): registers are full.
 // range: the ranges of tile rows of the group's planes, from plane 0 of the
 // strip buffer.  err: bit 0 when a bounded wait ran out.
 // Bound: 32 planes of 4096^2 take 1.22 ms, the sum of the column factor (1.21)
@@ -540,8 +537,8 @@ template <int N>
 __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
     k_colimage(StackArgs a, const float2* __restrict__ tw1, const float2* __restrict__ tw2,
                const int2* __restrict__ range, int log2T, const float4* __restrict__ strips, ScreenTab tab,
-               float2* __restrict__ acc, const double* __restrict__ sum_w, void* image, int units,
-               unsigned long long* __restrict__ err)
+               float2* __restrict__ part, float2* __restrict__ acc, const double* __restrict__ sum_w, void* image,
+               int units, unsigned long long* __restrict__ err)
 {
     constexpr int r = N / 256, kPer = N / 16, S = strips_per_block<N>(), kThreads = col_threads<N>();
     constexpr int kUnits = N / 2 / S;  // units per channel
@@ -554,7 +551,7 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
     unsigned long long* full = reinterpret_cast<unsigned long long*>(s2 + 15 * r);
     __shared__ int s_abort;
 
-    const int t = threadIdx.x, nk = a.nk, slots = nk + 2;
+    const int t = threadIdx.x, nk = a.nk;
     const ColThread<N> me(t);
     const unsigned long long limit = a.wait_ns ? a.wait_ns : kStripWaitNs;
     if (t == 0) {
@@ -564,21 +561,26 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
     }
     __syncthreads();
 
-    // thread 0: issue the next slot in order (unit iu, slot is of it), if any
-    int iu = blockIdx.x, is = 0, ist = 0, issued = 0;
+    // whether plane p of the group is the first of its run (or of the group)
+    auto run_start = [&](int p) { return p == 0 || (a.k0 + p) % kScreenRun == 0; };
+    // thread 0: issue the next slot in order, if any: of unit iu the rho rows (ip
+    // = nk), plane ip, or the fin rows after it (ifin)
+    int iu = blockIdx.x, ip = nk, ist = 0, issued = 0;
+    bool ifin = false;
     auto issue = [&]() {
         if (iu >= units) return;
         const int chan = iu / kUnits, strip0 = (iu - chan * kUnits) * S;
         const uint32_t bar = smem_u32(full + ist);
         float4* dst = stage + (size_t)ist * S * N;
-        if (is == 0 || is == nk + 1) {
-            const float2* src = is ? tab.fin : tab.rho;
+        if (ip == nk || ifin) {
+            const float2* src = ifin ? tab.fin : tab.rho;
+            const int table = ifin ? (a.chan0 + chan) * tab.runs + (a.k0 + ip) / kScreenRun : a.chan0 + chan;
             mbar_expect(bar, S * 2 * kRow * (uint32_t)sizeof(float2));
             for (int q = 0; q < 2 * S; ++q)
                 bulk_load(smem_u32(reinterpret_cast<float2*>(dst + (q >> 1) * N) + (q & 1) * kRow),
-                          src + screen_row<N>(a.chan0 + chan, 2 * strip0 + q), kRow * (uint32_t)sizeof(float2), bar);
-        } else if (is != a.skip_slot1) {
-            const int p = a.plane0 + chan * nk + nk - is;
+                          src + screen_row<N>(table, 2 * strip0 + q), kRow * (uint32_t)sizeof(float2), bar);
+        } else if (nk - ip != a.skip_slot1) {
+            const int p = a.plane0 + chan * nk + ip;
             const int2 rg = __ldg(range + p);
             const uint32_t row0 = (uint32_t)rg.x << log2T, bytes = ((uint32_t)(rg.y - rg.x) << log2T) * 16u;
             mbar_expect(bar, S * bytes);
@@ -589,8 +591,13 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
         }
         ++issued;
         if (++ist == kStripStages) ist = 0;
-        if (++is == slots) {
-            is = 0;
+        if (ip < nk && !ifin && run_start(ip)) {
+            ifin = true;
+            return;
+        }
+        ifin = false;
+        if (--ip < 0) {
+            ip = nk;
             iu += gridDim.x;
         }
     };
@@ -631,7 +638,7 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
 
     for (int u = blockIdx.x; u < units; u += gridDim.x) {
         const int chan = u / kUnits, strip0 = (u - chan * kUnits) * S;
-        const int plane0 = a.plane0 + chan * nk, x = 2 * (strip0 + me.sub) + me.c;
+        const int plane0 = a.plane0 + chan * nk, px = 2 * (strip0 + me.sub) + me.c;
         float2 rho[16], h[16];
         {
             const float2* row = wait() + me.c * kRow;
@@ -644,78 +651,95 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
             next();
         }
         bool bad = false;
-        for (int p = nk - 1; p >= 0; --p) {
-            const int2 rg = __ldg(range + plane0 + p);
-            // rows j + kPer q of the range: q from qlo to qhi - 1
-            const int qlo = ((rg.x << log2T) + kPer - 1 - me.j) / kPer, qhi = ((rg.y << log2T) + kPer - 1 - me.j) / kPer;
-            const uint32_t in = (1u << qhi) - (1u << qlo);
-            float2* buf = wait() + me.c;
-            cpx x[16];
+        for (int phi = nk; phi > 0 && !bad;) {
+            // the run [plo, phi)
+            const int plo = max(0, (a.k0 + phi - 1) / kScreenRun * kScreenRun - a.k0);
+            for (int p = phi - 1; p >= plo; --p) {
+                const int2 rg = __ldg(range + plane0 + p);
+                // rows j + kPer q of the range: q from qlo to qhi - 1
+                const int qlo = ((rg.x << log2T) + kPer - 1 - me.j) / kPer, qhi = ((rg.y << log2T) + kPer - 1 - me.j) / kPer;
+                const uint32_t in = (1u << qhi) - (1u << qlo);
+                float2* buf = wait() + me.c;
+                cpx x[16];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                x[q] = cpx_make(0.f, 0.f);
-                if (in & (1u << q)) x[q] = lds_c(buf + 2 * (me.j + kPer * q));
+                for (int q = 0; q < 16; ++q) {
+                    x[q] = cpx_make(0.f, 0.f);
+                    if (in & (1u << q)) x[q] = lds_c(buf + 2 * (me.j + kPer * q));
+                }
+                if (r == 4) __syncwarp();  // pos1 moves values between neighbouring lanes
+                dft16<1>(x);
+                sts_c(buf + 2 * pos1<N>(0, me.j), x[0]);
+#pragma unroll
+                for (int q = 1; q < 16; ++q) sts_c(buf + 2 * pos1<N>(q, me.j), c_mul(x[q], w1[(q - 1) * kPer]));
+                if (!barrier()) {
+                    bad = true;
+                    break;
+                }
+#pragma unroll
+                for (int b = 0; b < 16; ++b) x[b] = lds_c(buf + 2 * pos1<N>(me.k1, me.g + r * b));
+                __syncwarp();  // the block's reads (pos1) before its writes (pos2)
+                dft16<1>(x);
+                sts_c(buf + 2 * pos2<N>(me.k1, 0, me.g), x[0]);
+#pragma unroll
+                for (int k2 = 1; k2 < 16; ++k2) sts_c(buf + 2 * pos2<N>(me.k1, k2, me.g), c_mul(x[k2], w2[(k2 - 1) * r]));
+                __syncwarp();
+#pragma unroll
+                for (int ii = 0; ii < 16 / r; ++ii) {
+                    cpx y[r];
+#pragma unroll
+                    for (int q = 0; q < r; ++q) y[q] = lds_c(buf + 2 * pos2<N>(me.k1, me.g + r * ii, q));
+                    dft_small<r, 1>(y);
+#pragma unroll
+                    for (int k3 = 0; k3 < r; ++k3) {
+                        const int o = ii * r + k3;
+                        const float2 v = cpx_get(y[k3]), g = h[o];
+                        h[o].x = fmaf(g.x, rho[o].x, fmaf(-g.y, rho[o].y, v.x));
+                        h[o].y = fmaf(g.x, rho[o].y, fmaf(g.y, rho[o].x, v.y));
+                    }
+                }
+                next();
             }
-            if (r == 4) __syncwarp();  // pos1 moves values between neighbouring lanes
-            dft16<1>(x);
-            sts_c(buf + 2 * pos1<N>(0, me.j), x[0]);
+            if (bad) break;
+            // a group that begins within a run: on to the run's first plane
+            for (int z = (a.k0 + plo) % kScreenRun; z > 0; --z) {
 #pragma unroll
-            for (int q = 1; q < 16; ++q) sts_c(buf + 2 * pos1<N>(q, me.j), c_mul(x[q], w1[(q - 1) * kPer]));
+                for (int o = 0; o < 16; ++o) h[o] = c_mul(h[o], rho[o]);
+            }
+            const float2* row = wait() + me.c * kRow;
             if (!barrier()) {
                 bad = true;
                 break;
             }
+            const bool top = phi == nk;  // the unit's first run
+            float2* mine = part + (size_t)blockIdx.x * 16 * kThreads + t;
+            const int ch = a.chan_screen ? a.chan0 + chan : 0;
+            const double sw = sum_w[ch];
+            const float inv_sw = (sw != 0.0) ? (float)(1.0 / sw) : 0.0f;
+            float* out = reinterpret_cast<float*>(image) + (size_t)ch * a.img_stride;
 #pragma unroll
-            for (int b = 0; b < 16; ++b) x[b] = lds_c(buf + 2 * pos1<N>(me.k1, me.g + r * b));
-            __syncwarp();  // the block's reads (pos1) before its writes (pos2)
-            dft16<1>(x);
-            sts_c(buf + 2 * pos2<N>(me.k1, 0, me.g), x[0]);
-#pragma unroll
-            for (int k2 = 1; k2 < 16; ++k2) sts_c(buf + 2 * pos2<N>(me.k1, k2, me.g), c_mul(x[k2], w2[(k2 - 1) * r]));
-            __syncwarp();
-            if (p + 1 < nk && (p + 1) % kStripResync == 0) {
-                const float2* row = tab.kap + screen_row<N>(a.chan0 + chan, 2 * (strip0 + me.sub) + me.c);
-#pragma unroll
-                for (int o = 0; o < 16; ++o) h[o] = c_mul(h[o], __ldg(row + me.entry(o)));
-            }
-#pragma unroll
-            for (int ii = 0; ii < 16 / r; ++ii) {
-                cpx y[r];
-#pragma unroll
-                for (int q = 0; q < r; ++q) y[q] = lds_c(buf + 2 * pos2<N>(me.k1, me.g + r * ii, q));
-                dft_small<r, 1>(y);
-#pragma unroll
-                for (int k3 = 0; k3 < r; ++k3) {
-                    const int o = ii * r + k3;
-                    const float2 v = cpx_get(y[k3]), g = h[o];
-                    h[o].x = fmaf(g.x, rho[o].x, fmaf(-g.y, rho[o].y, v.x));
-                    h[o].y = fmaf(g.x, rho[o].y, fmaf(g.y, rho[o].x, v.y));
+            for (int o = 0; o < 16; ++o) {
+                const int y = me.y(o);
+                const int64_t pix = (int64_t)y * N + px;
+                float2 v = c_mul(h[o], row[me.entry(o)]);
+                h[o] = make_float2(0.f, 0.f);
+                if (!top) v = c_add(v, mine[o * kThreads]);
+                if (plo > 0) {
+                    mine[o * kThreads] = v;
+                    continue;
                 }
+                if ((px + y) & 1) v = make_float2(-v.x, -v.y);  // fftshift sign
+                if (!a.first) v = c_add(v, acc[pix]);
+                if (!a.last)
+                    acc[pix] = v;
+                else if (a.flags & RICK_REAL_IMAGE)
+                    out[pix] = v.x * inv_sw;
+                else
+                    reinterpret_cast<float2*>(out)[pix] = make_float2(v.x * inv_sw, v.y * inv_sw);
             }
             next();
+            phi = plo;
         }
         if (bad) break;
-        const float2* row = wait() + me.c * kRow;
-        if (!barrier()) break;
-        const int ch = a.chan_screen ? a.chan0 + chan : 0;
-        const double sw = sum_w[ch];
-        const float inv_sw = (sw != 0.0) ? (float)(1.0 / sw) : 0.0f;
-        float* out = reinterpret_cast<float*>(image) + (size_t)ch * a.img_stride;
-#pragma unroll
-        for (int o = 0; o < 16; ++o) {
-            const int y = me.y(o);
-            const int64_t pix = (int64_t)y * N + x;
-            float2 v = c_mul(h[o], row[me.entry(o)]);
-            if ((x + y) & 1) v = make_float2(-v.x, -v.y);  // fftshift sign
-            if (!a.first) v = c_add(v, acc[pix]);
-            if (!a.last)
-                acc[pix] = v;
-            else if (a.flags & RICK_REAL_IMAGE)
-                out[pix] = v.x * inv_sw;
-            else
-                reinterpret_cast<float2*>(out)[pix] = make_float2(v.x * inv_sw, v.y * inv_sw);
-        }
-        next();
     }
     if (!ok) s_abort = 1;
     __syncthreads();
@@ -736,7 +760,8 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
 // Adjoint of k_colimage: for every plane of the group, the rows of its range
 // of the (forward) column transforms of R conj(screen), R the adjoint of the
 // finalisation applied to the image gradient, in strip order.  The pixels'
-// conjugate rotation advances the screened value from plane to plane.  Planes
+// conjugate rotation advances the screened value from plane to plane within a
+// run of planes, whose first value is made from the pixels again.  Planes
 // alternate between two exchange buffers, so that the barrier between passes 2
 // and 1 of a plane also covers the reads of the plane before.  32 planes of
 // 4096^2: 1.48 ms, 0.94 ms with the rows after it (0.26 of the tiles written):
@@ -765,47 +790,50 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
     // the table rows of the block's columns, through shared memory
     constexpr int kRow = N / 2 + 16;
     float2* rows = reinterpret_cast<float2*>(strip_smem) + (size_t)(2 * me.sub + me.c) * kRow;
-    auto load_rows = [&](const float2* src) {
+    auto load_rows = [&](const float2* src, int table) {
         __syncthreads();
         for (int i = t; i < 2 * S * kRow; i += kThreads) {
             const int col = i / kRow;
-            reinterpret_cast<float2*>(strip_smem)[i] = __ldg(src + screen_row<N>(0, 2 * blockIdx.x * S + col) + i - col * kRow);
+            reinterpret_cast<float2*>(strip_smem)[i] = __ldg(src + screen_row<N>(table, 2 * blockIdx.x * S + col) + i - col * kRow);
         }
         __syncthreads();
     };
-    load_rows(tab.rho);
+    load_rows(tab.rho, 0);
 #pragma unroll
     for (int o = 0; o < 16; ++o) {
         rho[o] = rows[me.entry(o)];
         rho[o].y = -rho[o].y;
     }
-    load_rows(tab.fin);
+    // the screened values of plane p: the run's first plane's, rotated on to it
+    auto start = [&](int p) {
+        const int run = (a.k0 + p) / kScreenRun;
+        load_rows(tab.fin, run);
 #pragma unroll
-    for (int o = 0; o < 16; ++o) {
-        const int y = me.y(o);
-        const int64_t pix = (int64_t)y * N + x0;
-        float2 z = rows[me.entry(o)];
-        const float s = ((x0 + y) & 1) ? -inv_sw : inv_sw;  // fftshift sign
-        z = make_float2(z.x * s, -z.y * s);
-        const float2 v = (a.flags & RICK_REAL_IMAGE) ? make_float2(reinterpret_cast<const float*>(rimg)[pix], 0.f)
-                                                     : reinterpret_cast<const float2*>(rimg)[pix];
-        q[o] = c_mul(v, z);
-    }
-    __syncthreads();
+        for (int o = 0; o < 16; ++o) {
+            const int y = me.y(o);
+            const int64_t pix = (int64_t)y * N + x0;
+            float2 z = rows[me.entry(o)];
+            const float s = ((x0 + y) & 1) ? -inv_sw : inv_sw;  // fftshift sign
+            z = make_float2(z.x * s, -z.y * s);
+            const float2 v = (a.flags & RICK_REAL_IMAGE) ? make_float2(reinterpret_cast<const float*>(rimg)[pix], 0.f)
+                                                         : reinterpret_cast<const float2*>(rimg)[pix];
+            q[o] = c_mul(v, z);
+        }
+        __syncthreads();
+        for (int z = (a.k0 + p) - run * kScreenRun; z > 0; --z) {
+#pragma unroll
+            for (int o = 0; o < 16; ++o) q[o] = c_mul(q[o], rho[o]);
+        }
+    };
 
     float2* dst0 = reinterpret_cast<float2*>(strips + (size_t)(blockIdx.x * S + me.sub) * N) + me.c;
     int which = 0;
     for (int p = 0; p < a.nk; ++p) {
         const int2 rg = __ldg(range + p);
         const int vlo = rg.x << log2T, vhi = rg.y << log2T;
-        if (p > 0) {
-            if (p % kStripResync == 0) {
-#pragma unroll
-                for (int o = 0; o < 16; ++o) {
-                    const float2 d = __ldg(tab.kap + screen_row<N>(0, x0) + me.entry(o));
-                    q[o] = c_mul(q[o], make_float2(d.x, -d.y));
-                }
-            }
+        if (p == 0 || (a.k0 + p) % kScreenRun == 0) {
+            start(p);
+        } else {
 #pragma unroll
             for (int o = 0; o < 16; ++o) q[o] = c_mul(q[o], rho[o]);
         }
@@ -910,8 +938,8 @@ cudaError_t launch_colimage_n(const StripArgs& s, const StackArgs& a, const floa
     const int units = nchan * (N / 2 / strips_per_block<N>());
     const int resident = sm_count_strip() * (512 / col_threads<N>());
     k_colimage<N><<<(unsigned)std::min(units, resident), col_threads<N>(), colimage_smem<N>(), st>>>(
-        a, s.tw1, s.tw2, s.range + s.k0, s.log2T, reinterpret_cast<const float4*>(strips), s.tab, acc, sum_w, image,
-        units, err);
+        a, s.tw1, s.tw2, s.range + s.k0, s.log2T, reinterpret_cast<const float4*>(strips), s.tab, s.part, acc, sum_w,
+        image, units, err);
     return cudaGetLastError();
 }
 
@@ -974,15 +1002,17 @@ cudaError_t launch_rows(int n, int dir, const StripArgs& s, int k0, int nk, floa
     }
 }
 
-cudaError_t launch_screen(const StripArgs& s, const StackArgs& a, const float* taper, bool with_rho, int nchan,
-                          cudaStream_t st)
+cudaError_t launch_screen(const StripArgs& s, const StackArgs& a, const float* taper, int nchan, cudaStream_t st)
 {
-    if (nchan < 1 || nchan > 65535) return cudaErrorInvalidValue;
+    const int64_t tables = (int64_t)nchan * s.tab.runs;
+    if (nchan < 1 || tables < 1 || tables > 65535) return cudaErrorInvalidValue;
     const int side = a.n / 2 + 1;
-    k_screen<<<dim3((unsigned)((side + 255) / 256), (unsigned)side, (unsigned)nchan), 256, 0, st>>>(a, taper, s.tab,
-                                                                                                   with_rho ? 1 : 0);
+    k_screen<<<dim3((unsigned)((side + 255) / 256), (unsigned)side, (unsigned)tables), 256, 0, st>>>(a, taper, s.tab);
     return cudaGetLastError();
 }
+
+// k_colimage's `part`: 16 values of each thread that is resident (512 per SM).
+size_t strip_part_bytes(int runs) { return runs > 1 ? (size_t)sm_count_strip() * 512 * 16 * sizeof(float2) : 0; }
 
 cudaError_t launch_colimage(const StripArgs& s, const StackArgs& a, const float2* strips, float2* acc,
                             const double* sum_w, void* image, unsigned long long* err, cudaStream_t st, int nchan)
