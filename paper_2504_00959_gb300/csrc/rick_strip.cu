@@ -720,7 +720,9 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
             for (int o = 0; o < 16; ++o) {
                 const int y = me.y(o);
                 const int64_t pix = (int64_t)y * N + px;
-                float2 v = c_mul(h[o], row[me.entry(o)]);
+                const float2 f = row[me.entry(o)];
+                // outside the sky (f = 0) the pixel is 0 whatever the planes hold, infinities too
+                float2 v = f.x != 0.f || f.y != 0.f ? c_mul(h[o], f) : make_float2(0.f, 0.f);
                 h[o] = make_float2(0.f, 0.f);
                 if (!top) v = c_add(v, mine[o * kThreads]);
                 if (plo > 0) {
