@@ -319,6 +319,8 @@ struct PhaseScope {
 };
 
 void count_launches(rick_handle h, int64_t n) { h->timer.launches += n; }
+// the counting sort: count, scan and scatter
+int sort_launches(int64_t ntiles) { return 2 + scan_launches(ntiles); }
 
 void resolve_timer(rick_handle h, bool accumulate)
 {
@@ -1003,7 +1005,7 @@ rick_status rick_grid(rick_handle h, const float* vis, const float* u, const flo
     }
     h->chunks.push_back(ch);
     h->bytes_held += off_bytes + ent_bytes;
-    count_launches(h, 5);
+    count_launches(h, sort_launches(ntiles));
     return RICK_OK;
 }
 
@@ -1144,7 +1146,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
     if (e == cudaSuccess) e = launch_scan(h->cursor, ntiles, c.cstride, off, h->cursor, h->block_sums, h->stream);
     if (e == cudaSuccess) e = launch_primary_scatter(c, u, v, w, weights, nvis, density, h->cursor, perm, with_entries, h->stream);
     if (e != cudaSuccess) st = fail(h, RICK_ERR_CUDA, "rick_degrid sort: %s", cudaGetErrorString(e));
-    if (!st) count_launches(h, 5);
+    if (!st) count_launches(h, sort_launches(ntiles));
     // the adjoint of rick_fft_and_stack's transform path: with the strip
     // transform k_colspread, then the row transforms of the needed tiles; with the split,
     // k_spreadcol writes the planes after the adjoint of the last column
@@ -1472,7 +1474,7 @@ static rick_status batch_body(rick_handle h, const float* vis, const float* u, c
         RICK_CU(h, launch_scan(h->cursor, ntiles, c.cstride, h->b_off, h->cursor, h->block_sums, h->stream));
         RICK_CU(h, launch_scatter(c, u, v, w, weights, vis2, m, nullptr, h->cursor, h->b_ent, h->ctr, h->chan_sw,
                                   h->stream));
-        count_launches(h, 5);
+        count_launches(h, sort_launches(ntiles));
         if (h->strip || h->longrows) {
             ChunkList cl{};
             cl.off[0] = h->b_off;
@@ -1693,8 +1695,9 @@ rick_status rick_image_batch(rick_handle h, const float* vis, const float* u, co
         // per plane group the two gridder kernels, then k_colfft and one
         // k_colstack over its channels (split) or one k_stack over them
         const int groups = (c.nw + h->G - 1) / h->G;
-        count_launches(h, h->strip ? 6 + 4 * groups
-                                   : h->longrows ? 6 + 5 * groups : 5 + (h->batch_split ? 4 : 3) * groups);
+        const int sort = sort_launches((int64_t)c.nw * c.ntp);
+        count_launches(h, sort + (h->strip ? 1 + 4 * groups
+                                           : h->longrows ? 1 + 5 * groups : (h->batch_split ? 4 : 3) * groups));
         return RICK_OK;
     }
     if (!use_graph) return batch_body(h, vis, u, v, w, weights, m, images);

@@ -244,6 +244,7 @@ cudaError_t launch_count(const GridCfg& c, const float* u, const float* v, const
                          cudaStream_t s);
 // counts[i * stride] for i < len -> offsets[0..len] (packed, exclusive, total
 // last) and cursor[i * stride] = offsets[i]; counts may alias cursor
+int scan_launches(int64_t len);  // kernels that launch_scan launches
 cudaError_t launch_scan(const uint32_t* counts, int64_t len, int stride, uint32_t* offsets, uint32_t* cursor,
                         uint32_t* block_sums, cudaStream_t s);
 // chan_sw: per-channel weight sums (NULL: ctr->sum_w, single channel)

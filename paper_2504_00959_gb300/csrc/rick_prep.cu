@@ -843,6 +843,8 @@ cudaError_t launch_count(const GridCfg& c, const float* u, const float* v, const
     return cudaGetLastError();
 }
 
+int scan_launches(int64_t len) { return len <= 0 ? 0 : len <= kScanMax ? 1 : 3; }
+
 cudaError_t launch_scan(const uint32_t* counts, int64_t len, int stride, uint32_t* offsets, uint32_t* cursor,
                         uint32_t* block_sums, cudaStream_t s)
 {
