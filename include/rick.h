@@ -131,7 +131,8 @@ rick_status rick_destroy(rick_handle h);
  * default stream). */
 rick_status rick_set_stream(rick_handle h, void* cuda_stream);
 
-/* Device bytes rick_create + one rick_grid of max_vis measurements need. */
+/* Device bytes rick_create + one rick_grid of max_vis measurements need (with
+ * the second plane buffer of rick_fft_and_stack where the problem takes it). */
 rick_status rick_workspace_size(const rick_params* p, int64_t max_vis, size_t* bytes);
 
 /* Forget all gridded measurements, weight sums, counters and the uniform-

@@ -230,6 +230,49 @@ bool want_longrows(const rick_params& p) { return longrow_shape(p.n) && own_tran
 // keeps its order of summation too.
 constexpr double kGatherAmp = 1e5;
 
+// I0(x) by its power series (all terms positive); beyond binary64 it is infinite.
+double bessel_i0(double x)
+{
+    const double q = 0.25 * x * x;
+    double term = 1.0, sum = 1.0;
+    for (int k = 1; k < 2000 && term > 1e-17 * sum; ++k) {
+        term *= q / ((double)k * k);
+        sum += term;
+    }
+    return sum;
+}
+
+// mean(1 / c^2) of the taper without a device, for rick_workspace_size: c by
+// Simpson's rule in FP64 (512 intervals over the kernel; by symmetry half of
+// them and of the pixels), cos(t_i x) by its recurrence in i.
+double taper_amp(const GridCfg& c, double kparam)
+{
+    constexpr int kHalf = 256;
+    const double h = 0.5 * c.S / kHalf;
+    double g[kHalf + 1], den = 0.0;
+    for (int i = 0; i <= kHalf; ++i) {
+        const double t = i * h, z = 2.0 * t / c.S;
+        const double v = c.kernel == RICK_KERNEL_GAUSS
+                             ? std::exp(-t * t / (2.0 * kparam * kparam))
+                             : bessel_i0(kparam * std::sqrt(std::fmax(0.0, 1.0 - z * z)));
+        g[i] = v * (i == 0 || i == kHalf ? 1.0 : (i & 1) ? 4.0 : 2.0);
+        den += g[i];
+    }
+    double s2 = 0.0;
+    for (int x = 0; x <= c.n / 2; ++x) {  // pixel n / 2 - x: x = n / 2 occurs once, x = 0 once, the others twice
+        const double step = 2.0 * std::cos(6.283185307179586476925 * h * x / c.n);
+        double c0 = 1.0, c1 = 0.5 * step, num = g[0];
+        for (int i = 1; i <= kHalf; ++i) {
+            num += g[i] * c1;
+            const double c2 = step * c1 - c0;
+            c0 = c1;
+            c1 = c2;
+        }
+        s2 += (x == 0 || x == c.n / 2 ? 1.0 : 2.0) * (den / num) * (den / num);
+    }
+    return s2 / c.n;
+}
+
 rick_status get_plan(rick_handle h, int batch, cufftHandle* out, int kind = kPlan2D)
 {
     const int key = (kind << 24) | batch;
@@ -594,7 +637,7 @@ rick_status rick_workspace_size(const rick_params* p, int64_t max_vis, size_t* b
     b += (size_t)entries_bound(c, max_vis) * sizeof(float4);         // entries
     b += heavy_words_for(entries_bound(c, max_vis)) * sizeof(uint32_t);  // gridder's heavy-tile list
     if (p->flags & RICK_UNIFORM_WEIGHT) b += (size_t)c.n * c.n * sizeof(uint32_t);
-    if (want_strip(*p))  // the strip order's copy of a group, tile bits, row ranges, twiddles, screen
+    if (want_strip(*p) && (!(p->flags & RICK_GRID_CORRECT) || taper_amp(c, kp) <= kStripAmp))  // the strip order's copy of a group, tile bits, row ranges, twiddles, screen
         b += (size_t)G * plane_bytes(p) + (size_t)c.nw * (c.ntu * ((c.ntu + 31) / 32) + 2) * sizeof(uint32_t) +
              (size_t)15 * (c.n / 16 + c.n / 256) * sizeof(float2) + screen_bytes(c.n, screen_runs(c.nw)) +
              (c.nw > kScreenRun ? (size_t)160 * 512 * 16 * sizeof(float2) : 0);  // partial sums of at most 160 SMs
