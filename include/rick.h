@@ -170,8 +170,8 @@ rick_status rick_add_density(rick_handle h, const float* vis, const float* u, co
  * point) column factor of every plane of the group in place, and one the
  * last 16-point column factor together with the screen and the sum.
  * Otherwise, and with RICK_FFT_2D, cuFFT's 2D plan and a separate
- * screen-and-sum pass.  Where the second buffer would take more than half of
- * the device memory that is free, and where the grid correction amplifies rounding by more
+ * screen-and-sum pass.  Where the second buffer would take more than a quarter
+ * of the device memory that is free, and where the grid correction amplifies rounding by more
  * than 300 (mean of 1 / taper^2; support 8 or a Gaussian of 6 and wider),
  * n = 2048 and 4096 take the split and n = 1024 the 2D plan. */
 rick_status rick_fft_and_stack(rick_handle h, float* image);

@@ -203,8 +203,10 @@ bool use_split(const rick_params& p, int* n1, int* n2)
 // x 1e7 measurements 4.99 -> 3.52 ms per image, 8 channels of 2048^2 x 16
 // 5.70 -> 4.08 ms, 1024^2 x 16 x 1e6 0.358 -> 0.301 ms (0.343 without the scan in
 // one launch and the gridder's smaller blocks).  It needs a second buffer of a
-// group's planes (strip order); where that would take more than half of the
-// free memory, the handle takes the split transform or the 2D plan instead.
+// group's planes (strip order); where that would take more than a quarter of
+// the memory that is free beside the planes, the handle takes the split
+// transform or the 2D plan instead: what the program allocates afterwards finds
+// at least three quarters of what it would without the buffer.
 bool own_transform(const rick_params& p) { return !(p.flags & (RICK_FFT_2D | RICK_FFT_SPLIT)); }
 bool want_strip(const rick_params& p) { return strip_shape(p.n) && own_transform(p); }
 
@@ -494,9 +496,9 @@ bool strip_alloc(rick_handle h, bool strip)
     const size_t tab_bytes = strip ? h->nchan * screen_bytes(n, runs) : 0, strip_bytes = strip ? (size_t)h->G * pb : 0;
     const size_t part_bytes = strip ? strip_part_bytes(runs) : 0;
     const size_t need = strip_bytes + bits + rng + tw + tab_bytes + part_bytes;
-    // at most half of what is free: the rest is for the sorted measurements,
-    // whose number is not known yet
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || 2 * need + (64u << 20) > fr) return false;
+    // at most a quarter of what is free: the rest is for the sorted measurements,
+    // whose number is not known yet, and for other handles
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || 4 * need + (64u << 20) > fr) return false;
     std::vector<float2> w(tw / sizeof(float2));
     for (int k = 1; k < 16; ++k) {
         for (int j = 0; j < n / 16; ++j) {
@@ -735,12 +737,19 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
     int G = p->plane_group ? p->plane_group : NW;
     if (G > NW) G = NW;
     if (!p->plane_group) {
-        // planes + cuFFT's work area or the strip buffer: the 2D plan may need
-        // as much as the planes, the split transform's row plan far less
+        // planes + cuFFT's work area: the 2D plan may need as much as the
+        // planes, the split transform's row plan far less
         int n1 = 0, n2 = 0;
-        const bool split = !h->batch && use_split(*p, &n1, &n2) && !(want_strip(*p) && h->amp <= kStripAmp);
-        const size_t fit = split ? (size_t)(0.7 * (double)fr) / (pb ? pb : 1)
-                                 : (size_t)(0.6 * (double)fr) / (pb ? 2 * pb : 1);
+        const bool split = !h->batch && use_split(*p, &n1, &n2);
+        size_t fit = split ? (size_t)(0.7 * (double)fr) / (pb ? pb : 1)
+                           : (size_t)(0.6 * (double)fr) / (pb ? 2 * pb : 1);
+        // the strip transform where its groups (a seventh of the memory: planes,
+        // a batch's second buffer, and the strips in a quarter of the rest) hold
+        // a run of planes or everything; with smaller ones the former's
+        // larger groups
+        const size_t strips = fr / (7 * pb);
+        if (want_strip(*p) && h->amp <= kStripAmp && strips >= (size_t)std::min(NW, std::max(kScreenRun, c.nw_chan)))
+            fit = std::min(fit, strips);
         if ((size_t)G > fit) G = (int)(fit > 0 ? fit : 1);
         // groups of equal size (no short last group)
         const int ngroups = (NW + G - 1) / G;
