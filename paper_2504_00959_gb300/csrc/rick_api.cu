@@ -212,24 +212,31 @@ bool want_strip(const rick_params& p) { return strip_shape(p.n) && own_transform
 
 // Grid correction multiplies the planes' rounding (~3e-7 of their RMS,
 // uncorrelated between pixels) by 1 / (c(x) c(y)), over the image by mean(1 /
-// c^2) in RMS: 167 for the Kaiser-Bessel kernel of support 7, 479 for support
-// 8, 800 for the Gaussian of support 6 and over 1e6 for wider Gaussians, whose
-// transform passes through zero inside the image.  Two transforms that round
-// differently then differ by that much: of the image, 7e-6 at 167 and 2e-5 at
-// 479 (6 planes of 4096^2, 3e4 measurements).  Up to kStripAmp the image is
-// well above its rounding whatever the transform; beyond, a handle keeps the
-// transform that it always had, so that its images stay the same.
+// c^2) in RMS: 162 for the Kaiser-Bessel kernel of support 7, 462 for support 8,
+// 1350 for support 9, 774 for the Gaussian of support 6 and over 1e6 for wider
+// Gaussians, whose transform passes through zero inside the image.  Two
+// transforms that round differently then give images that differ by that much
+// (2048^2 x 16 planes: 6.8e-6, 1.8e-5, 4.9e-5, 2.7e-5 of the image).  None of them
+// is the more exact one: against FP64 the strip transform, the split and the 2D
+// plan are off by 6.16e-5, 6.17e-5, 6.17e-5 at support 7, 7.21e-5, 7.27e-5,
+// 7.34e-5 at 9 and 9.3e-4, 9.5e-4, 9.7e-4 at 12.  The limit keeps the result from
+// depending on what else is in memory: whether a handle has the strip buffer
+// depends on what is free when it is made, and up to kStripAmp that moves its
+// image by less than 1e-5.
 constexpr double kStripAmp = 300.0;
 // The split transform's rows of n = 8192 and 16384 over what is not empty
-// (rick_longrow.cu) round differently in one factor of three only: up to the
-// Kaiser-Bessel kernel of support 8.  16384^2 x 16 planes x 2.5e7 measurements
-// 47.5 -> 41.4 ms (gridding 6.8 -> 4.9, rows 18.3 -> 13.6), 8192^2 x 4 x 3e4 2.76
-// -> 2.40 ms.
+// (rick_longrow.cu) need a few MB, so they are there on any handle up to
+// kLongAmp, which holds the difference to cuFFT's rows (RICK_FFT_SPLIT) to 2e-5
+// of the image (8192^2 x 4: 7.6e-6 at support 7, 2.0e-5 at 8, 5.6e-5 at 9; the
+// errors against FP64 agree to three digits).  16384^2 x 16 planes x 2.5e7
+// measurements 47.5 -> 41.4 ms (gridding 6.8 -> 4.9, rows 18.3 -> 13.6), 8192^2 x 4
+// x 3e4 2.76 -> 2.40 ms.
 constexpr double kLongAmp = 600.0;
 bool want_longrows(const rick_params& p) { return longrow_shape(p.n) && own_transform(p); }
 // The adjoint's footprints, of planes that hold the corrected image, cancel by
-// the same factors: where they cancel by more than binary32 holds, the gather
-// keeps its order of summation too.
+// the same factors: where they cancel by more than binary32 holds, the order of
+// summation shows in the result, which is then row by row for lists of any
+// length.
 constexpr double kGatherAmp = 1e5;
 
 // I0(x) by its power series (all terms positive); beyond binary64 it is infinite.
@@ -639,7 +646,8 @@ rick_status rick_workspace_size(const rick_params* p, int64_t max_vis, size_t* b
     b += (size_t)entries_bound(c, max_vis) * sizeof(float4);         // entries
     b += heavy_words_for(entries_bound(c, max_vis)) * sizeof(uint32_t);  // gridder's heavy-tile list
     if (p->flags & RICK_UNIFORM_WEIGHT) b += (size_t)c.n * c.n * sizeof(uint32_t);
-    if (want_strip(*p) && (!(p->flags & RICK_GRID_CORRECT) || taper_amp(c, kp) <= kStripAmp))  // the strip order's copy of a group, tile bits, row ranges, twiddles, screen
+    // the strip order's copy of a group, tile bits, row ranges, twiddles, screen
+    if (want_strip(*p) && (!(p->flags & RICK_GRID_CORRECT) || taper_amp(c, kp) <= kStripAmp))
         b += (size_t)G * plane_bytes(p) + (size_t)c.nw * (c.ntu * ((c.ntu + 31) / 32) + 2) * sizeof(uint32_t) +
              (size_t)15 * (c.n / 16 + c.n / 256) * sizeof(float2) + screen_bytes(c.n, screen_runs(c.nw)) +
              (c.nw > kScreenRun ? (size_t)160 * 512 * 16 * sizeof(float2) : 0);  // partial sums of at most 160 SMs

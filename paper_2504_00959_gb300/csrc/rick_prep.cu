@@ -669,9 +669,10 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_add(const uint32_t* __restr
 // `cursor` may be the same array: every thread reads its counters before it
 // writes them, and neither pointer is declared free of aliases.
 // The sort of 1e5 measurements into 512 tiles took 35 us with three launches
-// for the scan and takes 28 with one; 1e6 into 16384 tiles 85 and 78.  Eight
-// SMs fall behind beyond: 5e5 into 32768 tiles 53.5 and 47.8, into 65536 54.6 and
-// 54.3, into 105300 and 131072 54.8 and 65.
+// for the scan and takes 28 with one.  Eight SMs fall behind beyond kScanMax: the
+// sort of 5e5 with three launches and with one takes 51 and 44.5 us for 16384
+// tiles, 50.4 and 44 for 32768, 50.5 and 50 for 49152, 50.4 and 50.3 for 65536, and
+// took 54.8 and 65 for 105300 and 131072.
 constexpr int kScanCluster = 8;
 constexpr int kScanSub = 2;  // tiles of kScanTile counters per CTA at most
 constexpr int64_t kScanMax = (int64_t)kScanCluster * kScanSub * kScanTile;

@@ -766,8 +766,10 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
 // run of planes, whose first value is made from the pixels again.  Planes
 // alternate between two exchange buffers, so that the barrier between passes 2
 // and 1 of a plane also covers the reads of the plane before.  32 planes of
-// 4096^2: 1.48 ms, 0.94 ms with the rows after it (0.26 of the tiles written):
-// together 2.4 where the adjoint stack, column factor and cuFFT's rows took 3.6.
+// 4096^2: 1.38 ms, the rows after it 0.91 (0.26 of the tiles written): together
+// 2.3 where the adjoint stack, column factor and cuFFT's rows took 3.6.  Bound by
+// latency: issue slots 39 % busy, the shared-memory pipe 43 %, at 16 warps per SM
+// (registers).
 template <int N>
 __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
     k_colspread(StackArgs a, const float2* __restrict__ tw1, const float2* __restrict__ tw2,
