@@ -700,10 +700,14 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
                 next();
             }
             if (bad) break;
-            // a group that begins within a run: on to the run's first plane
-            for (int z = (a.k0 + plo) % kScreenRun; z > 0; --z) {
+            // a group that begins within a run: on to the run's first plane, by
+            // the rotation's powers (the unit needs rho no more)
+            for (int z = (a.k0 + plo) % kScreenRun; z > 0; z >>= 1) {
 #pragma unroll
-                for (int o = 0; o < 16; ++o) h[o] = c_mul(h[o], rho[o]);
+                for (int o = 0; o < 16; ++o) {
+                    if (z & 1) h[o] = c_mul(h[o], rho[o]);
+                    rho[o] = c_mul(rho[o], rho[o]);
+                }
             }
             const float2* row = wait() + me.c * kRow;
             if (!barrier()) {
@@ -802,12 +806,15 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
         }
         __syncthreads();
     };
-    load_rows(tab.rho, 0);
+    auto load_rho = [&]() {
+        load_rows(tab.rho, 0);
 #pragma unroll
-    for (int o = 0; o < 16; ++o) {
-        rho[o] = rows[me.entry(o)];
-        rho[o].y = -rho[o].y;
-    }
+        for (int o = 0; o < 16; ++o) {
+            rho[o] = rows[me.entry(o)];
+            rho[o].y = -rho[o].y;
+        }
+    };
+    load_rho();
     // the screened values of plane p: the run's first plane's, rotated on to it
     auto start = [&](int p) {
         const int run = (a.k0 + p) / kScreenRun;
@@ -823,11 +830,16 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
                                                          : reinterpret_cast<const float2*>(rimg)[pix];
             q[o] = c_mul(v, z);
         }
-        __syncthreads();
-        for (int z = (a.k0 + p) - run * kScreenRun; z > 0; --z) {
+        const int from = (a.k0 + p) - run * kScreenRun;  // > 0: a group that begins within a run
+        for (int z = from; z > 0; z >>= 1) {
 #pragma unroll
-            for (int o = 0; o < 16; ++o) q[o] = c_mul(q[o], rho[o]);
+            for (int o = 0; o < 16; ++o) {
+                if (z & 1) q[o] = c_mul(q[o], rho[o]);
+                rho[o] = c_mul(rho[o], rho[o]);
+            }
         }
+        if (from > 0) load_rho();
+        __syncthreads();
     };
 
     float2* dst0 = reinterpret_cast<float2*>(strips + (size_t)(blockIdx.x * S + me.sub) * N) + me.c;
