@@ -20,6 +20,11 @@
 namespace rick {
 namespace {
 
+__device__ __forceinline__ bool aligned_to(const void* p, size_t bytes)
+{
+    return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) == 0;
+}
+
 constexpr int kStackThreads = 256;
 constexpr int kResync = 8;
 
@@ -112,10 +117,23 @@ __global__ void __launch_bounds__(kStackThreads) k_stack(StackArgs a_in, const f
         f0 /= wcorr_at(a, s0.nm1);
         f1 /= wcorr_at(a, s1.nm1);
     }
+    // the caller's image may be aligned to its elements only
     if (a.flags & RICK_REAL_IMAGE) {
-        reinterpret_cast<float2*>(image)[pix >> 1] = make_float2(a0.x * f0, a1.x * f1);
+        float* out = reinterpret_cast<float*>(image) + pix;
+        if (aligned_to(image, sizeof(float2))) {
+            *reinterpret_cast<float2*>(out) = make_float2(a0.x * f0, a1.x * f1);
+        } else {
+            out[0] = a0.x * f0;
+            out[1] = a1.x * f1;
+        }
     } else {
-        reinterpret_cast<float4*>(image)[pix >> 1] = make_float4(a0.x * f0, a0.y * f0, a1.x * f1, a1.y * f1);
+        float2* out = reinterpret_cast<float2*>(image) + pix;
+        if (aligned_to(image, sizeof(float4))) {
+            *reinterpret_cast<float4*>(out) = make_float4(a0.x * f0, a0.y * f0, a1.x * f1, a1.y * f1);
+        } else {
+            out[0] = make_float2(a0.x * f0, a0.y * f0);
+            out[1] = make_float2(a1.x * f1, a1.y * f1);
+        }
     }
 }
 
@@ -140,11 +158,15 @@ __global__ void __launch_bounds__(kStackThreads) k_spread(StackArgs a, const voi
     PixelScreen s0 = pixel_screen(a, x0, y), s1 = pixel_screen(a, x0 + 1, y);
     float2 r0, r1;
     if (a.flags & RICK_REAL_IMAGE) {
-        const float2 rr = reinterpret_cast<const float2*>(rimg)[pix >> 1];
+        const float* in = reinterpret_cast<const float*>(rimg) + pix;
+        const float2 rr = aligned_to(rimg, sizeof(float2)) ? *reinterpret_cast<const float2*>(in)
+                                                           : make_float2(in[0], in[1]);
         r0 = make_float2(rr.x, 0.f);
         r1 = make_float2(rr.y, 0.f);
     } else {
-        const float4 rr = reinterpret_cast<const float4*>(rimg)[pix >> 1];
+        const float2* in = reinterpret_cast<const float2*>(rimg) + pix;
+        const float4 rr = aligned_to(rimg, sizeof(float4)) ? *reinterpret_cast<const float4*>(in)
+                                                           : make_float4(in[0].x, in[0].y, in[1].x, in[1].y);
         r0 = make_float2(rr.x, rr.y);
         r1 = make_float2(rr.z, rr.w);
     }
