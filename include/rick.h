@@ -177,7 +177,8 @@ rick_status rick_add_density(rick_handle h, const float* vis, const float* u, co
 rick_status rick_fft_and_stack(rick_handle h, float* image);
 
 /* Eq. 3 alone: the gridded planes k0 .. k0+nk-1 as complex float
- * [nk][n][n] (no fftshift sign), fully overwritten. */
+ * [nk][n][n] (no fftshift sign), fully overwritten; 16-byte aligned
+ * (RICK_ERR_ARG otherwise). */
 rick_status rick_grid_planes(rick_handle h, int32_t k0, int32_t nk, float* planes);
 
 /* Adjoint of the measurement-to-image map (degridding; not in the paper):
@@ -305,6 +306,7 @@ rick_status rick_set_prep_blocks(rick_handle h, int32_t blocks_per_sm);
  * and 64 bytes per measurement (16 when support is 1), each piece 256-byte
  * aligned -- must fit in those 64 MiB; otherwise RICK_ERR_ARG before any
  * launch, with the reason written to err (err_len bytes; err may be NULL).
+ * planes is 16-byte aligned (RICK_ERR_ARG otherwise).
  * All calls on a device share the array and it keeps the last call's
  * contents, so calls whose GPU work overlaps race: the caller must order
  * them.  The first call on a device, and the first for each kernel

@@ -1076,6 +1076,8 @@ rick_status rick_grid_planes(rick_handle h, int32_t k0, int32_t nk, float* plane
     if (k0 < 0 || nk < 0 || k0 + nk > h->p.nw) return fail(h, RICK_ERR_ARG, "plane range out of bounds");
     if (nk == 0) return RICK_OK;
     if (!planes) return fail(h, RICK_ERR_ARG, "planes is NULL");
+    if (reinterpret_cast<uintptr_t>(planes) % sizeof(float4))  // the gridder stores pairs of cells
+        return fail(h, RICK_ERR_ARG, "planes must be 16-byte aligned");
     return grid_pass(h, k0, nk, false, reinterpret_cast<float2*>(planes), true);
 }
 

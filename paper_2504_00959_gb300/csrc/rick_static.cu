@@ -90,6 +90,10 @@ extern "C" rick_status rick_grid_planes_static(const rick_params* p, const float
         set_msg(err, err_len, "planes, vis, u, v, w must not be NULL");
         return RICK_ERR_ARG;
     }
+    if (reinterpret_cast<uintptr_t>(planes) % sizeof(float4)) {  // the gridder stores pairs of cells
+        set_msg(err, err_len, "planes must be 16-byte aligned");
+        return RICK_ERR_ARG;
+    }
     cudaStream_t stream = (cudaStream_t)cuda_stream;
 
     // scratch layout: counters | coefficients | cursor (+1 word) | offsets | scan sums | density | entries
