@@ -173,7 +173,9 @@ rick_status rick_add_density(rick_handle h, const float* vis, const float* u, co
  * screen-and-sum pass.  Where the second buffer would take more than a quarter
  * of the device memory that is free, and where the grid correction amplifies rounding by more
  * than 300 (mean of 1 / taper^2; support 8 or a Gaussian of 6 and wider),
- * n = 2048 and 4096 take the split and n = 1024 the 2D plan. */
+ * n = 2048 and 4096 take the split and n = 1024 the 2D plan; so do single
+ * images in several groups of fewer than 4 planes each, and n = 1024 with
+ * fewer than 12 planes in a group. */
 rick_status rick_fft_and_stack(rick_handle h, float* image);
 
 /* Eq. 3 alone: the gridded planes k0 .. k0+nk-1 as complex float

@@ -224,6 +224,19 @@ bool want_strip(const rick_params& p) { return strip_shape(p.n) && own_transform
 // depends on what is free when it is made, and up to kStripAmp that moves its
 // image by less than 1e-5.
 constexpr double kStripAmp = 300.0;
+// Whether single images of NW planes in groups of G take the strip transform.
+// Its column kernel reads two rows of screen tables per column, and adds to the
+// sum of the groups before, once per group: groups of few planes are faster by
+// the former transform (the split, 2D plan at n = 1024), former / strip time of
+// images and of adjoints over a track's and a disk's coverage, 48 planes:
+// 4096^2 in groups of 1 plane .82-.86 and .95-1.02, of 2 .90-.98 and 1.01-1.10, of 3
+// .94-1.05 and 1.04-1.15, of 4 1.02-1.15 and 1.08-1.22; 2048^2 of 1 .71-.74 and
+// .95-1.05, 3 .97-1.07 and 1.02-1.15, 4 1.02-1.17 and 1.09-1.22; 1024^2 of 8 .91-1.01
+// and .86-.99, 12 1.05-1.18 and .97-1.11.  A single group of 1 to 3 planes has the
+// whole image to gain from the fused stack at 2048^2 (1.10-1.24 and .92-1.06) and
+// 4096^2 (1.25-1.36 and .98-1.10), not at 1024^2 (8 planes .97-1.03 and .86-.96).
+bool strip_pays(int n, int G, int NW) { return n == 1024 ? G >= 12 : G >= 4 || G == NW; }
+
 // The split transform's rows of n = 8192 and 16384 over what is not empty
 // (rick_longrow.cu) need a few MB, so they are there on any handle up to
 // kLongAmp, which holds the difference to cuFFT's rows (RICK_FFT_SPLIT) to 2e-5
@@ -647,7 +660,7 @@ rick_status rick_workspace_size(const rick_params* p, int64_t max_vis, size_t* b
     b += heavy_words_for(entries_bound(c, max_vis)) * sizeof(uint32_t);  // gridder's heavy-tile list
     if (p->flags & RICK_UNIFORM_WEIGHT) b += (size_t)c.n * c.n * sizeof(uint32_t);
     // the strip order's copy of a group, tile bits, row ranges, twiddles, screen
-    if (want_strip(*p) && (!(p->flags & RICK_GRID_CORRECT) || taper_amp(c, kp) <= kStripAmp))
+    if (want_strip(*p) && strip_pays(p->n, G, p->nw) && (!(p->flags & RICK_GRID_CORRECT) || taper_amp(c, kp) <= kStripAmp))
         b += (size_t)G * plane_bytes(p) + (size_t)c.nw * (c.ntu * ((c.ntu + 31) / 32) + 2) * sizeof(uint32_t) +
              (size_t)15 * (c.n / 16 + c.n / 256) * sizeof(float2) + screen_bytes(c.n, screen_runs(c.nw)) +
              (c.nw > kScreenRun ? (size_t)160 * 512 * 16 * sizeof(float2) : 0);  // partial sums of at most 160 SMs
@@ -756,7 +769,8 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
         // a run of planes or everything; with smaller ones the former's
         // larger groups
         const size_t strips = fr / (7 * pb);
-        if (want_strip(*p) && h->amp <= kStripAmp && strips >= (size_t)std::min(NW, std::max(kScreenRun, c.nw_chan)))
+        if (want_strip(*p) && h->amp <= kStripAmp && (h->batch || strip_pays(p->n, NW, NW)) &&
+            strips >= (size_t)std::min(NW, std::max(kScreenRun, c.nw_chan)))
             fit = std::min(fit, strips);
         if ((size_t)G > fit) G = (int)(fit > 0 ? fit : 1);
         // groups of equal size (no short last group)
@@ -882,7 +896,7 @@ static rick_status create_impl(const rick_params* p, int nchan, const double* w_
             for (int j = 0; j < kPolyTerms; ++j) h->cfg.coef[t][j] = (t < c.S) ? coef[t * kPolyTerms + j] : 0.0f;
         set_tap_sum(h->cfg);
     }
-    h->strip = want_strip(*p) && h->amp <= kStripAmp && strip_alloc(h, true);
+    h->strip = want_strip(*p) && h->amp <= kStripAmp && (h->batch || strip_pays(p->n, G, NW)) && strip_alloc(h, true);
     h->longrows = want_longrows(*p) && h->amp <= kLongAmp && strip_alloc(h, false);
     // the cuFFT plans this handle's transform path uses
     if (!h->strip) {

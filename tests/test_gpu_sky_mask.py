@@ -8,7 +8,7 @@ import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,nw", [(1024, 3), (1024, 40), (2048, 2), (4096, 2), (8192, 2)])
+@pytest.mark.parametrize("n,nw", [(1024, 13), (1024, 40), (2048, 2), (4096, 2), (8192, 2)])
 def test_overflowing_planes(n, nw):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")

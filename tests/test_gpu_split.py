@@ -33,7 +33,7 @@ def _same(a, b, tol):
     assert (a - b).abs().max().item() <= tol * b.abs().max().item()
 
 
-@pytest.mark.parametrize("n,nw,extra", [(1024, 8, {}), (2048, 5, {"plane_group": 2}), (4096, 33, {}), (8192, 3, {})])
+@pytest.mark.parametrize("n,nw,extra", [(1024, 16, {}), (2048, 9, {"plane_group": 4}), (4096, 33, {}), (8192, 3, {})])
 def test_single(rick, n, nw, extra):
     prob = synth.config2(m=100000, n=n, nw=nw)
     g = {k: prob[k].cuda() for k in ("vis", "u", "v", "w", "wt")}

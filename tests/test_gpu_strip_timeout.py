@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 REAL = synth.FLAG_REAL
 
 
-@pytest.mark.parametrize("n,nw,slot", [(1024, 8, 0), (1024, 40, 21), (2048, 5, 4), (4096, 3, 1)])
+@pytest.mark.parametrize("n,nw,slot", [(1024, 12, 0), (1024, 40, 21), (2048, 5, 4), (4096, 3, 1)])
 def test_times_out_and_recovers(n, nw, slot):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
