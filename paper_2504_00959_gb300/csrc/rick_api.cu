@@ -1193,7 +1193,7 @@ static rick_status degrid_impl(rick_handle h, const GridCfg& c, const double* su
     RICK_CU(h, cudaMemGetInfo(&fr, &tot));
     fr += pool_idle(h);  // this call's scratch takes again what an earlier one's left in the pool
     // the sorted measurements where they fit, else their indices
-    const bool by_rows = !(h->amp <= kGatherAmp) || !gather_by_columns(c, nvis);
+    const bool by_rows = !(h->amp <= kGatherAmp) || !gather_by_columns(c, nvis * std::min(h->G, c.nw) / c.nw);
     bool with_entries = !by_rows && off_bytes + primary_list_bytes(nvis, true) + (64u << 20) <= fr;
     if (off_bytes + primary_list_bytes(nvis, with_entries) + (64u << 20) > fr)
         return fail(h, RICK_ERR_OOM, "degrid scratch does not fit");

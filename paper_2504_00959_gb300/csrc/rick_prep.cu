@@ -774,14 +774,17 @@ cudaError_t launch_gather_s(const GridCfg& c, const PrimaryList& list, const uin
 }
 
 // Whether k_degrid_gather (a lane per footprint column) is to gather m
-// measurements, and k_degrid_gather_rows otherwise: supports that fill its
-// groups of 4 or 8 lanes, and lists that fill the chip's warps, each of which
-// takes 32 measurements one group step after another.  Predictions, row by row
-// and by columns, us: support 8 at 2000^2 x 8 planes, 5e4 measurements 350 and 349, 3e5
-// 378 and 374, 6e6 973 and 861, at 512^2 5e4 71 and 79, 3e5 97 and 96, 6e6 771 and 681;
-// support 4 at 2000^2 6e6 785 and 693.  Lanes without a column cost what the
-// kernel gains: support 6 at 512^2, 3e5 85 and 100, 6e6 610 and 631; support 9 at
-// 2000^2 6e6 1069 and 1184; support 12 1403 and 1350 there, but 411 and 432 at 3e5.
+// measurements per launch (a plane group's share of a call's), and
+// k_degrid_gather_rows otherwise: supports that fill its groups of 4 or 8 lanes,
+// and lists that fill the chip's warps, each of which takes 32 measurements one
+// group step after another.  Predictions, row by row and by columns, us: support
+// 8 at 2000^2 x 8 planes, 5e4 measurements 350 and 349, 3e5 378 and 374, 6e6 973
+// and 861, at 512^2 5e4 71 and 79, 3e5 97 and 96, 6e6 771 and 681; support 4 at
+// 2000^2 6e6 785 and 693.  Lanes without a column cost what the kernel gains:
+// support 6 at 512^2, 3e5 85 and 100, 6e6 610 and 631; support 9 at 2000^2 6e6 1069
+// and 1184; support 12 1403 and 1350 there, but 411 and 432 at 3e5.  Per launch:
+// 1.1e6 measurements of support 7 at 256^2 x 43 planes take 403 and 485 in groups
+// of 3 planes (7.7e4 each), 148 by columns and 158 by rows in one.
 bool gather_by_columns(const GridCfg& c, int64_t m)
 {
     return (c.S == 4 || c.S == 7 || c.S == 8) && m >= ((int64_t)1 << 18);
