@@ -45,10 +45,14 @@ constexpr uint32_t kHeavyMin = 64;
 constexpr uint32_t kHeavyMax = 768;
 constexpr uint32_t kHeavyDiv = 16384;
 // Tiles a warp of k_grid_tiles takes: as many as leave every SM kTileWarps
-// warps, between one and kTilesPerWarp.  A run of tiles shares staging rounds
-// and hides their list reads, but with eight each the 4096 tiles of 16 planes of
-// 512^2 made 128 blocks of four warps, less than one per SM (gridding 163 -> 139
-// us with one each; 16 planes of 1024^2 137 -> 128, 12 of 1000^2 100 -> 92).
+// warps, a power of two between one and kTilesPerWarp.  A run of tiles shares
+// staging rounds and hides their list reads, but with eight each the 4096 tiles
+// of 16 planes of 512^2 made 128 blocks of four warps, less than one per SM
+// (gridding 163 -> 152 us with one each; 16 planes of 1024^2 146 -> 119 with two,
+// 12 of 1000^2 103 -> 95).  Powers of two keep a block's tiles from straddling
+// the rows of tiles, whose middle holds the entries: two chunks of 4e5, dense at
+// the centre, on 2 planes of 2048^2 in tiles of 16 take 500 us with eight, 525
+// with six, 455 with four.
 constexpr int kTilesPerWarp = 8;
 constexpr int kTileWarps = 32;
 
@@ -914,7 +918,8 @@ cudaError_t launch_grid_s(const GridCfg& c, const ChunkList& ch, int k0, int nk,
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(heavy, 0, 4 * sizeof(uint32_t), s)) != cudaSuccess) return e;
     const int64_t fit = ntl / ((int64_t)sm_count_grid() * kTileWarps);
-    const int tpw = (int)std::min<int64_t>(std::max<int64_t>(fit, 1), kTilesPerWarp);
+    int tpw = 1;
+    while (2 * tpw <= fit && tpw < kTilesPerWarp) tpw *= 2;
     const unsigned tile_blocks = (unsigned)((nblocks + tpw - 1) / tpw);
     k_grid_tiles<S><<<tile_blocks, 32 * wl, tile_bytes * wl, s>>>(c, ch, k0, ntl, shift ? 1 : 0, accumulate ? 1 : 0,
                                                                   skip_empty ? 1 : 0, tpw, planes, hl);
