@@ -490,6 +490,7 @@ void strip_free(rick_handle h)
     cudaFree(h->strips);
     cudaFree(h->sargs.bits);
     cudaFree(h->sargs.range);
+    cudaFree(h->sargs.occ);
     cudaFree(h->sargs.tab.rho);
     cudaFree(h->sargs.part);
     cudaFree(const_cast<float2*>(h->sargs.tw1));
@@ -510,12 +511,13 @@ bool strip_alloc(rick_handle h, bool strip)
     const int n = h->p.n, r = n / 256, wpr = (c.ntu + 31) / 32;
     size_t fr = 0, tot = 0;
     const size_t bits = (size_t)c.nw * c.ntu * wpr * sizeof(uint32_t), rng = (size_t)c.nw * sizeof(int2);
+    const size_t occ = (size_t)c.nw * sizeof(int4);
     const int q = strip ? 0 : n / 4096;
     const size_t t1 = 15 * (size_t)(n / 16), t2 = 15 * (size_t)r, tw = (t1 + t2 + 15 * (size_t)q) * sizeof(float2);
     const int runs = screen_runs(c.nw_chan);
     const size_t tab_bytes = strip ? h->nchan * screen_bytes(n, runs) : 0, strip_bytes = strip ? (size_t)h->G * pb : 0;
     const size_t part_bytes = strip ? strip_part_bytes(runs) : 0;
-    const size_t need = strip_bytes + bits + rng + tw + tab_bytes + part_bytes;
+    const size_t need = strip_bytes + bits + rng + occ + tw + tab_bytes + part_bytes;
     // at most a quarter of what is free: the rest is for the sorted measurements,
     // whose number is not known yet, and for other handles
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || 4 * need + (64u << 20) > fr) return false;
@@ -538,6 +540,8 @@ bool strip_alloc(rick_handle h, bool strip)
     bool ok = (!strip || cudaMalloc((void**)&h->strips, strip_bytes) == cudaSuccess) &&
               cudaMalloc((void**)&h->sargs.bits, bits) == cudaSuccess &&
               cudaMalloc((void**)&h->sargs.range, rng) == cudaSuccess &&
+              cudaMalloc((void**)&h->sargs.occ, occ) == cudaSuccess &&
+              cudaMemset(h->sargs.occ, 0, occ) == cudaSuccess &&
               (!strip || cudaMalloc((void**)&h->sargs.tab.rho, tab_bytes) == cudaSuccess) &&
               (!part_bytes || cudaMalloc((void**)&h->sargs.part, part_bytes) == cudaSuccess) &&
               cudaMalloc((void**)&dev_tw, tw) == cudaSuccess;
@@ -661,7 +665,7 @@ rick_status rick_workspace_size(const rick_params* p, int64_t max_vis, size_t* b
     if (p->flags & RICK_UNIFORM_WEIGHT) b += (size_t)c.n * c.n * sizeof(uint32_t);
     // the strip order's copy of a group, tile bits, row ranges, twiddles, screen
     if (want_strip(*p) && strip_pays(p->n, G, p->nw) && (!(p->flags & RICK_GRID_CORRECT) || taper_amp(c, kp) <= kStripAmp))
-        b += (size_t)G * plane_bytes(p) + (size_t)c.nw * (c.ntu * ((c.ntu + 31) / 32) + 2) * sizeof(uint32_t) +
+        b += (size_t)G * plane_bytes(p) + (size_t)c.nw * (c.ntu * ((c.ntu + 31) / 32) + 6) * sizeof(uint32_t) +
              (size_t)15 * (c.n / 16 + c.n / 256) * sizeof(float2) + screen_bytes(c.n, screen_runs(c.nw)) +
              (c.nw > kScreenRun ? (size_t)160 * 512 * 16 * sizeof(float2) : 0);  // partial sums of at most 160 SMs
     b += plane_bytes(p);                                             // cuFFT work area (estimate)

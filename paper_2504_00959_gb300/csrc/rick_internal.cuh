@@ -355,6 +355,7 @@ struct ScreenTab {
 struct StripArgs {
     uint32_t* bits;
     int2* range;
+    int4* occ;  // k_occupancy's maxima per plane, zero between launches
     int wpr, log2T, k0;
     const float2* tw1;
     const float2* tw2;

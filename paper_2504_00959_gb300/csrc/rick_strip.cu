@@ -59,18 +59,24 @@ int sm_count_strip()
 
 constexpr int kOccThreads = 1024;
 constexpr int kOccBatch = 8;
+constexpr int kOccWords = kOccThreads / 32 * kOccBatch;
 
-// One block per plane: the plane's tile bits (wpr words per tile row) and its
-// range of non-empty tile rows [lo, hi).  Lists: a tile is non-empty when any
+// grid (parts, planes): the plane's tile bits (wpr words per tile row) and its
+// range of non-empty tile rows [lo, hi).  A block takes kOccWords words, all of a
+// plane up to n = 2048 with tiles of 32; of several blocks the last to finish
+// writes the range, from maxima in `occ` (which it leaves zero again).  With one
+// block per plane, planes of 4096^2, 8192^2 and 16384^2 took 12, 34 and 118 us (16,
+// 49 and 185 in the adjoint); now 9 (11) each, the offsets' latency.  Lists: a tile is non-empty when any
 // of them has entries there.  Adjoint (reach > 0, one list, sorted by the tile
 // of the first footprint cell on the first plane of the w-footprint): a tile
 // of plane k is needed when it or its left, upper or upper left neighbour
 // holds a measurement of the planes k - reach + 1 .. k.
 __global__ void __launch_bounds__(kOccThreads) k_occupancy(GridCfg c, ChunkList ch, int reach, int wpr,
-                                                           uint32_t* __restrict__ bits, int2* __restrict__ range)
+                                                           uint32_t* __restrict__ bits, int2* __restrict__ range,
+                                                           int4* __restrict__ occ)
 {
     __shared__ int s_lo, s_hi;
-    const int k = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int k = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
         s_lo = c.ntu;
         s_hi = 0;
@@ -78,9 +84,10 @@ __global__ void __launch_bounds__(kOccThreads) k_occupancy(GridCfg c, ChunkList 
     __syncthreads();
     const int words = c.ntu * wpr;
     int lo = c.ntu, hi = 0;
-    // kOccBatch words per trip: their first list's offsets are in flight together
+    // kOccBatch words per warp: their first list's offsets are in flight together
     constexpr int kWarps = kOccThreads / 32;
-    for (int i0 = wid; i0 < words; i0 += kOccBatch * kWarps) {
+    {
+        const int i0 = blockIdx.x * kOccWords + wid;
         uint32_t o0[kOccBatch], o1[kOccBatch];
 #pragma unroll
         for (int b = 0; b < kOccBatch; ++b) {
@@ -123,7 +130,23 @@ __global__ void __launch_bounds__(kOccThreads) k_occupancy(GridCfg c, ChunkList 
         atomicMax(&s_hi, hi);
     }
     __syncthreads();
-    if (threadIdx.x == 0) range[k] = s_hi > s_lo ? make_int2(s_lo, s_hi) : make_int2(0, 0);
+    if (threadIdx.x != 0) return;
+    if (gridDim.x == 1) {
+        range[k] = s_hi > s_lo ? make_int2(s_lo, s_hi) : make_int2(0, 0);
+        return;
+    }
+    int* o = reinterpret_cast<int*>(occ + k);  // tile rows from lo on, hi, blocks that are done
+    if (s_hi > s_lo) {
+        atomicMax(o, c.ntu - s_lo);
+        atomicMax(o + 1, s_hi);
+    }
+    __threadfence();
+    if (atomicAdd(o + 2, 1) == (int)gridDim.x - 1) {
+        __threadfence();
+        const int from = atomicExch(o, 0), to = atomicExch(o + 1, 0);
+        atomicExch(o + 2, 0);
+        range[k] = to > 0 ? make_int2(c.ntu - from, to) : make_int2(0, 0);
+    }
 }
 
 // ------------------------------------------------------------------- rows
@@ -1001,7 +1024,8 @@ bool strip_shape(int n) { return n == 1024 || n == 2048 || n == 4096; }
 
 cudaError_t launch_occupancy(const GridCfg& c, const ChunkList& ch, int reach, const StripArgs& s, cudaStream_t st)
 {
-    k_occupancy<<<(unsigned)c.nw, kOccThreads, 0, st>>>(c, ch, reach, s.wpr, s.bits, s.range);
+    const int parts = (c.ntu * s.wpr + kOccWords - 1) / kOccWords;
+    k_occupancy<<<dim3((unsigned)parts, (unsigned)c.nw), kOccThreads, 0, st>>>(c, ch, reach, s.wpr, s.bits, s.range, s.occ);
     return cudaGetLastError();
 }
 
