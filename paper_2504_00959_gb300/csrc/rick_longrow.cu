@@ -16,6 +16,7 @@
 // Blocks k1 lie at an odd pitch, and pass 3's half warps take q values of s and
 // every q-th block: all four passes read and write without bank conflicts.
 #include <algorithm>
+#include <atomic>
 
 #include "rick_dft.cuh"
 #include "rick_internal.cuh"
@@ -166,20 +167,22 @@ __global__ void __launch_bounds__(N / 16, N >= 16384 ? 1 : 2)
 template <int N, int DIR>
 cudaError_t launch_long_n(const StripArgs& s, int k0, int nk, int row_perm, float2* planes, cudaStream_t st)
 {
-    static bool done[64] = {};
-    static int sms[64] = {};
-    int dev = 0;
+    // SMs of a device, once its shared-memory opt-in is done (handles on several
+    // threads: written after both, read before either is relied on)
+    static std::atomic<int> ready[64];
+    int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) dev = 0;
-    if (!done[dev]) {
+    const bool known = dev >= 0 && dev < 64;
+    if (known) sms = ready[dev].load(std::memory_order_acquire);
+    if (!sms) {
         e = cudaFuncSetAttribute(k_longrows<N, DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)LongShape<N>::kSmem);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        done[dev] = true;
+        if (known) ready[dev].store(sms, std::memory_order_release);
     }
-    const dim3 grid((unsigned)(sms[dev] * (N >= 16384 ? 1 : 2)), (unsigned)nk);
+    const dim3 grid((unsigned)(sms * (N >= 16384 ? 1 : 2)), (unsigned)nk);
     const float2* tw3 = s.tw2 + 15 * LongShape<N>::r;
     k_longrows<N, DIR><<<grid, N / 16, LongShape<N>::kSmem, st>>>(s.tw1, s.tw2, tw3, s.bits, s.range, k0, s.wpr, s.log2T,
                                                                  row_perm, planes);

@@ -29,6 +29,7 @@
 // the DFT matrix is symmetric, so the same passes in reverse order (3, 2, 1)
 // also transform y to v, which k_colspread uses.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "rick_dft.cuh"
@@ -43,16 +44,15 @@ namespace {
 
 int sm_count_strip()
 {
-    static int cached[64] = {0};
-    int dev = 0;
+    static std::atomic<int> cached[64];
+    int dev = 0, v = 0;
     cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) dev = 0;
-    if (!cached[dev]) {
-        int v = 0;
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        cached[dev] = v > 0 ? v : 1;
-    }
-    return cached[dev];
+    const bool known = dev >= 0 && dev < 64;
+    if (known && (v = cached[dev].load(std::memory_order_relaxed)) > 0) return v;
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    v = v > 0 ? v : 1;
+    if (known) cached[dev].store(v, std::memory_order_relaxed);
+    return v;
 }
 
 // ------------------------------------------------------------- occupancy
@@ -924,14 +924,14 @@ __global__ void __launch_bounds__(col_threads<N>(), 512 / col_threads<N>())
 }
 
 template <typename K>
-cudaError_t opt_in(K kernel, size_t bytes, bool (&done)[64])
+cudaError_t opt_in(K kernel, size_t bytes, std::atomic<bool> (&done)[64])
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
+    if (dev >= 0 && dev < 64 && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
     return e;
 }
 
@@ -939,7 +939,7 @@ template <int N, int DIR, int LOG2T>
 cudaError_t launch_rows_n(const StripArgs& s, int k0, int nk, float2* planes, unsigned long long wait_ns,
                           unsigned long long* err, cudaStream_t st)
 {
-    static bool done[64] = {};
+    static std::atomic<bool> done[64];
     const cudaError_t e = opt_in(k_rows<N, DIR, LOG2T>, rows_smem<N>(), done);
     if (e != cudaSuccess) return e;
     // two blocks per SM and plane (a plane at a time); n = 4096 gives each several row groups
@@ -971,7 +971,7 @@ template <int N>
 cudaError_t launch_colimage_n(const StripArgs& s, const StackArgs& a, const float2* strips, float2* acc,
                               const double* sum_w, void* image, unsigned long long* err, int nchan, cudaStream_t st)
 {
-    static bool done[64] = {};
+    static std::atomic<bool> done[64];
     const cudaError_t e = opt_in(k_colimage<N>, colimage_smem<N>(), done);
     if (e != cudaSuccess) return e;
     const int units = nchan * (N / 2 / strips_per_block<N>());
@@ -986,7 +986,7 @@ template <int N>
 cudaError_t launch_colspread_n(const StripArgs& s, const StackArgs& a, const void* rimg, const double* sum_w,
                                float2* strips, cudaStream_t st)
 {
-    static bool done[64] = {};
+    static std::atomic<bool> done[64];
     const cudaError_t e = opt_in(k_colspread<N>, colspread_smem<N>(), done);
     if (e != cudaSuccess) return e;
     k_colspread<N><<<(unsigned)(N / 2 / strips_per_block<N>()), col_threads<N>(), colspread_smem<N>(), st>>>(
